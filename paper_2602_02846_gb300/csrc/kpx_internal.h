@@ -316,25 +316,29 @@ struct RefineParams {
     float* ckpt;            // [count][n_ckpt][REFINE_CKPT_WORDS]
     // broad phase of the box sum (null: every box at every step)
     struct RefineGridHeader* grid;
-    int32_t* grid_off;      // [REFINE_GRID_CELLS + 1]
+    int32_t* grid_off;      // [REFINE_GRID_CELLS + 1] (fewer at the coarse resolution)
+    int32_t* grid_cubes;    // [REFINE_GRID_CUBES]
     uint16_t* grid_ids;     // [REFINE_GRID_ENTRIES]
 };
 
-// The box grid of the refinement objective: a uniform grid of
-// REFINE_GRID_AXIS^3 cells over the boxes grown by the distance beyond which
-// a box's term is dropped; cell c lists, in index order, every box whose
-// grown box meets it.  Built on the device at each kpx_refine_eval call; the
-// counters count the box tests of the call's kernels.
-constexpr int REFINE_GRID_AXIS = 16;
-constexpr int REFINE_GRID_CELLS = REFINE_GRID_AXIS * REFINE_GRID_AXIS * REFINE_GRID_AXIS;
-constexpr int REFINE_GRID_ENTRIES = 1 << 22;
+// The box grid of the refinement objective: a uniform grid over the boxes
+// grown by the distance beyond which a box's term is dropped, of
+// REFINE_GRID_AXIS_MAX cells an axis or half as many; cell c lists, in index
+// order, every box that a point in it can reach.  Built on the device at each
+// kpx_refine_eval call; the counters count the box tests of the call's
+// kernels.  The offsets and the lists share a fixed part of the workspace.
+constexpr int REFINE_GRID_AXIS_MAX = 32;
+constexpr int REFINE_GRID_CELLS = REFINE_GRID_AXIS_MAX * REFINE_GRID_AXIS_MAX * REFINE_GRID_AXIS_MAX;
+constexpr size_t REFINE_GRID_BYTES = 256 + (size_t)(16 * 16 * 16 + 1) * 4 + ((size_t)1 << 22) * 2;
+constexpr int REFINE_GRID_CUBES = REFINE_GRID_CELLS / 64;  // of 4^3 cells, whose totals follow the offsets
+constexpr size_t REFINE_GRID_OFF_BYTES = ((size_t)(REFINE_GRID_CELLS + 1 + REFINE_GRID_CUBES) * 4 + 255) / 256 * 256;
+constexpr int REFINE_GRID_ENTRIES = (int)((REFINE_GRID_BYTES - 256 - REFINE_GRID_OFF_BYTES) / 2);
 struct RefineGridHeader {
     float lo[3], inv_cs[3];
-    int32_t ok, total;
+    int32_t axis, ok, total;
     unsigned long long tests[4];  // forward candidates, forward near, backward candidates, backward near
 };
 static_assert(sizeof(RefineGridHeader) <= 256, "the grid header's slot");
-constexpr size_t REFINE_GRID_BYTES = 256 + (size_t)(REFINE_GRID_CELLS + 1) * 4 + (size_t)REFINE_GRID_ENTRIES * 2;
 
 struct AdamParams {
     int32_t count, max_segments;

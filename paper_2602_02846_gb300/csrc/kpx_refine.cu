@@ -160,7 +160,8 @@ extern "C" kpx_status kpx_refine_eval(const kpx_dynamics* dyn, const kpx_refine_
         char* w = reinterpret_cast<char*>(workspace);
         R.grid = reinterpret_cast<RefineGridHeader*>(w);
         R.grid_off = reinterpret_cast<int32_t*>(w + 256);
-        R.grid_ids = reinterpret_cast<uint16_t*>(w + 256 + (size_t)(REFINE_GRID_CELLS + 1) * 4);
+        R.grid_cubes = R.grid_off + REFINE_GRID_CELLS + 1;
+        R.grid_ids = reinterpret_cast<uint16_t*>(w + 256 + REFINE_GRID_OFF_BYTES);
     }
     R.ckpt = workspace ? reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + grid_region()) : nullptr;
     return launch_refine_eval(R, reinterpret_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? KPX_OK : KPX_E_CUDA;
