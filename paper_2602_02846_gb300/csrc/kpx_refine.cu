@@ -14,12 +14,11 @@
 #include <cstring>
 
 #include "kpx_device.cuh"
+#include "kpx_refine.cuh"
 
 namespace kpx {
 
 namespace {
-
-constexpr int VAL_WARPS = 4;  // trajectories per block
 
 struct ValidateParams {
     int32_t count, max_segments, n_obs;
@@ -33,57 +32,296 @@ struct ValidateParams {
     float* x_end;
 };
 
-// one warp per trajectory: every lane integrates, the box tests are split
-// across the lanes
-__global__ void __launch_bounds__(VAL_WARPS * 32) k_refine_validate(DevParams P, ValidateParams V) {
-    extern __shared__ float smem[];
-    const int M = V.n_obs;
-    for (int i = threadIdx.x; i < 6 * M; i += blockDim.x) smem[i] = V.obs[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t tr = (int64_t)blockIdx.x * VAL_WARPS + (threadIdx.x >> 5);
-    if (tr >= V.count) return;
-    const int S = V.n_seg[tr];
-    float x[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) x[i] = V.x0[tr * 12 + i];
-    bool ok = S >= 0 && S <= V.max_segments;
-    // the edge costs of every segment, in FP64 from the FP32 controls:
-    // K h (1 + w e(u)); they do not depend on the states
-    double total = 0.0;
-    const double mg = (double)P.param[0] * (double)P.param[1];
-    const double tm = (double)P.param[5];
-    for (int s = 0; ok && s < S; ++s) {
-        const float* uv = V.u + (tr * V.max_segments + s) * 4;
-        const double et = ((double)uv[0] - mg) / mg;
-        const double e = et * et + ((double)uv[1] * uv[1] + (double)uv[2] * uv[2] + (double)uv[3] * uv[3]) / (tm * tm);
-        total += (double)V.steps[tr * V.max_segments + s] * (double)P.h * (1.0 + (double)P.w_effort * e);
+// A block takes up to 32 trajectories.  One warp integrates them, a lane
+// each, 32 steps at a time, leaving every state in shared memory; meanwhile
+// sixteen warps lay out the controls of the next 32 steps and check the states
+// of the previous ones (a trajectory a warp, a step a lane): bounds, then the
+// boxes of the point's cell in a grid that the block builds over the workspace
+// box.  The first state that fails ends its trajectory.  One more warp adds
+// the FP64 costs.  Bound: the longest trajectory's chain of RK4 steps, about
+// 400 cycles each.  With a warp per trajectory, every step waiting for its
+// 1,000 box tests (31 a lane), 512 sequences of up to 2,076 steps took 6.03
+// ms; this form takes 0.49 ms.
+constexpr int VAL_CHECK_WARPS = 16;
+constexpr int VAL_COST_WARP = 4;  // on one scheduler with the integrating warp 0, which so gets the fewest checkers
+constexpr int VAL_WARPS = VAL_CHECK_WARPS + 2;
+constexpr int VAL_PER_WARP = 32 / VAL_CHECK_WARPS;
+constexpr int VAL_ROW_BYTES = 2 * 32 * (int)(sizeof(float4) + sizeof(int) + 12 * sizeof(float));  // per trajectory
+constexpr int VAL_AXIS = 16;
+constexpr int VAL_CELLS = VAL_AXIS * VAL_AXIS * VAL_AXIS;
+constexpr int VAL_ENTRIES = 16384;
+constexpr int VAL_GRID_BYTES = VAL_CELLS * (int)sizeof(int) + VAL_ENTRIES * (int)sizeof(uint16_t);
+
+// the integrating and the checking warps, once per 32 steps
+__device__ __forceinline__ void validate_barrier() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"((VAL_CHECK_WARPS + 1) * 32) : "memory");
+}
+
+// The block's grid over the workspace box: cell c lists boxes
+// ids[c > 0 ? end[c - 1] : 0 .. end[c]), in any order.  The cell map is
+// monotone, so a point in the workspace and in a box lies in a cell that
+// lists the box.
+struct ValGrid {
+    int* end;
+    uint16_t* ids;
+    float inv[3];
+    bool ok;  // false: the lists do not fit, every box is tested
+
+    __device__ __forceinline__ int axis_cell(const DevParams& P, float v, int a) const {
+        return grid_cell(v, P.ws_lo[a], inv[a], VAL_AXIS);
     }
-    Stepper<KPX_QUAD12, KPX_RK4> st;
-    for (int s = 0; ok && s < S; ++s) {
-        const float4 uv = *reinterpret_cast<const float4*>(V.u + (tr * V.max_segments + s) * 4);
-        const float u[4] = {uv.x, uv.y, uv.z, uv.w};
-        const int K = V.steps[tr * V.max_segments + s];
-        st.init(P, x, u);
-        for (int k = 0; ok && k < K; ++k) {
-            st.advance(P, x, u);
-            bool hit = false;
-            for (int b = lane; b < M; b += 32) {
-                const float* o = smem + 6 * b;
-                hit |= x[0] >= o[0] && x[0] <= o[3] && x[1] >= o[1] && x[1] <= o[4] && x[2] >= o[2] && x[2] <= o[5];
+};
+
+template <bool SMEM_BOXES>
+__device__ __forceinline__ void box_of(const ValidateParams& V, const float4* s_box, int b, float4& lo, float4& hi) {
+    if constexpr (SMEM_BOXES) {
+        lo = s_box[2 * b];
+        hi = s_box[2 * b + 1];
+    } else {
+        const float* o = V.obs + 6 * b;
+        lo = make_float4(__ldg(o), __ldg(o + 1), __ldg(o + 2), 0.0f);
+        hi = make_float4(__ldg(o + 3), __ldg(o + 4), __ldg(o + 5), 0.0f);
+    }
+}
+
+// called by the whole block; a warp per box, its cells over the lanes
+template <bool SMEM_BOXES>
+__device__ void build_grid(const DevParams& P, const ValidateParams& V, const float4* s_box, ValGrid& G) {
+    __shared__ int s_warp[32];
+    __shared__ int s_total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float w = P.ws_hi[a] - P.ws_lo[a];
+        G.inv[a] = w > 0.0f ? (float)VAL_AXIS / w : 0.0f;
+    }
+    for (int c = threadIdx.x; c < VAL_CELLS; c += VAL_WARPS * 32) G.end[c] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {  // counts, then lists
+        for (int b = warp; b < V.n_obs; b += VAL_WARPS) {
+            float4 lo, hi;
+            box_of<SMEM_BOXES>(V, s_box, b, lo, hi);
+            const int x0 = G.axis_cell(P, lo.x, 0), y0 = G.axis_cell(P, lo.y, 1), z0 = G.axis_cell(P, lo.z, 2);
+            const int nx = max(G.axis_cell(P, hi.x, 0) - x0 + 1, 0), ny = max(G.axis_cell(P, hi.y, 1) - y0 + 1, 0),
+                      nz = max(G.axis_cell(P, hi.z, 2) - z0 + 1, 0);
+            for (int k = lane; k < nx * ny * nz; k += 32) {
+                const int c = ((z0 + k / (nx * ny)) * VAL_AXIS + y0 + k / nx % ny) * VAL_AXIS + x0 + k % nx;
+                const int pos = atomicAdd(&G.end[c], 1);  // second pass: from the cell's first entry on
+                if (pass == 1) G.ids[pos] = (uint16_t)b;
             }
-            ok = bounds_ok<12>(P, x) && !__any_sync(0xFFFFFFFFu, hit);
+        }
+        __syncthreads();
+        if (pass == 1) break;
+        // counts -> first entries (the second pass moves them to the ends)
+        constexpr int PER = VAL_CELLS / 512;
+        static_assert(VAL_WARPS * 32 >= 512, "512 threads scan the cells");
+        int v[PER], sum = 0;
+        const bool in = threadIdx.x < 512;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            v[q] = in ? G.end[threadIdx.x * PER + q] : 0;
+            sum += v[q];
+        }
+        int x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        int run = x - sum;
+        for (int w = 0; w < warp; ++w) run += s_warp[w];
+        if (threadIdx.x == VAL_WARPS * 32 - 1) s_total = run + sum;
+        if (in) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                G.end[threadIdx.x * PER + q] = run;
+                run += v[q];
+            }
+        }
+        __syncthreads();
+        G.ok = s_total <= VAL_ENTRIES;
+        if (!G.ok) return;
+    }
+}
+
+// whether a point of the workspace box lies in a box
+template <bool SMEM_BOXES>
+__device__ __forceinline__ bool in_a_box(const DevParams& P, const ValidateParams& V, const float4* s_box,
+                                         const ValGrid& G, float px, float py, float pz) {
+    int e0 = 0, e1 = V.n_obs;
+    if (G.ok) {
+        const int c = (G.axis_cell(P, pz, 2) * VAL_AXIS + G.axis_cell(P, py, 1)) * VAL_AXIS + G.axis_cell(P, px, 0);
+        e0 = c > 0 ? G.end[c - 1] : 0;
+        e1 = G.end[c];
+    }
+    bool hit = false;
+    for (int e = e0; e < e1 && !hit; ++e) {
+        float4 lo, hi;
+        box_of<SMEM_BOXES>(V, s_box, G.ok ? (int)G.ids[e] : e, lo, hi);
+        hit = px >= lo.x && px <= hi.x && py >= lo.y && py <= hi.y && pz >= lo.z && pz <= hi.z;
+    }
+    return hit;
+}
+
+template <bool ISO, bool SMEM_BOXES>
+__global__ void __launch_bounds__(VAL_WARPS * 32, 1) k_refine_validate(DevParams P, ValidateParams V, int per_block,
+                                                                      int row) {
+    extern __shared__ __align__(16) unsigned char val_smem[];
+    __shared__ long long s_total[32];
+    __shared__ int s_done[2][32];  // 1: ended, 2: ended by a state that is not valid
+    float4* su = reinterpret_cast<float4*>(val_smem);          // [chunk & 1][step][row]
+    float* sx = reinterpret_cast<float*>(su + 2 * 32 * row);   // [chunk & 1][component][step][row]
+    int* sseg = reinterpret_cast<int*>(sx + 2 * 12 * 32 * row);  // [chunk & 1][step][row]
+    ValGrid G;
+    G.end = sseg + 2 * 32 * row;
+    G.ids = reinterpret_cast<uint16_t*>(G.end + VAL_CELLS);
+    float4* s_box = reinterpret_cast<float4*>(val_smem + ((size_t)VAL_ROW_BYTES * row + VAL_GRID_BYTES));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * per_block;
+    const int nt = (int)min((int64_t)per_block, V.count - base);
+    if (SMEM_BOXES) {
+        float* f = reinterpret_cast<float*>(s_box);
+        for (int i = threadIdx.x; i < 6 * V.n_obs; i += VAL_WARPS * 32) {
+            const int b = i / 6, c = i - 6 * b;
+            f[8 * b + (c < 3 ? c : c + 1)] = V.obs[i];
         }
     }
-    if (ok) ok = in_goal(P, x[0], x[1], x[2]);
-    if (lane == 0) {
-        V.valid[tr] = ok ? 1 : 0;
-        V.cost[tr] = total;
-    }
-    if (V.x_end && lane < 12) {
+    for (int i = warp; i < 32; i += VAL_WARPS) {
+        long long t = -1;
+        const int S = i < nt ? V.n_seg[base + i] : -1;
+        if (S >= 0 && S <= V.max_segments) {
+            t = 0;
+            for (int s = lane; s < S; s += 32) t += segment_steps(V, base + i, S, s);
 #pragma unroll
-        for (int i = 0; i < 12; ++i)
-            if (lane == i) V.x_end[tr * 12 + i] = x[i];
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        }
+        if (lane == 0) {
+            s_total[i] = t;  // -1: no such trajectory, or a bad segment count
+            s_done[0][i] = s_done[1][i] = t > 0 ? 0 : 1;
+        }
+    }
+    __syncthreads();
+    if (V.n_obs > 0)
+        build_grid<SMEM_BOXES>(P, V, s_box, G);
+    else
+        G.ok = false;
+    const int64_t tr = base + lane;
+    if (warp == 0) {
+        float x[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) x[i] = lane < nt ? V.x0[tr * 12 + i] : 0.0f;
+        Stepper<KPX_QUAD12, KPX_RK4> st;
+        st.init(P, x, {});
+        int seg = -1;
+        long long left = s_total[lane];
+        validate_barrier();
+        for (int c = 0;; ++c) {  // chunk c; s_done[c & 1] as of the chunks before c - 1
+            const bool done = s_done[c & 1][lane] != 0;
+            if (__all_sync(0xFFFFFFFFu, done)) break;
+            const int here = done ? 0 : (int)(left < 32 ? left : 32);
+            left -= here;
+            const float4* uc = su + (c & 1) * 32 * row + lane;
+            const int* gs = sseg + (c & 1) * 32 * row + lane;
+            float* o = sx + (c & 1) * 12 * 32 * row + lane;
+            for (int t = 0; t < here; ++t) {
+                const float4 v = uc[t * row];
+                const float u[4] = {v.x, v.y, v.z, v.w};
+                const int s = gs[t * row];
+                if (s != seg) {  // a segment starts as the planner's rollouts do
+                    st.init(P, x, u);
+                    seg = s;
+                }
+                st.template advance<ISO ? 1 : 0>(P, x, u);
+#pragma unroll
+                for (int d = 0; d < 12; ++d) o[(d * 32 + t) * row] = x[d];
+            }
+            validate_barrier();
+        }
+        if (lane < nt && s_done[0][lane] != 2 && s_done[1][lane] != 2) {
+            V.valid[tr] = s_total[lane] >= 0 && in_goal(P, x[0], x[1], x[2]) ? 1 : 0;
+            if (V.x_end)
+#pragma unroll
+                for (int d = 0; d < 12; ++d) V.x_end[tr * 12 + d] = x[d];
+        }
+    } else if (warp == VAL_COST_WARP) {
+        // the edge costs of every segment, in FP64 from the FP32 controls:
+        // K h (1 + w e(u)); they do not depend on the states
+        if (lane < nt) {
+            double total = 0.0;
+            const double mg = (double)P.param[0] * (double)P.param[1];
+            const double tm = (double)P.param[5];
+            const int S = s_total[lane] >= 0 ? V.n_seg[tr] : 0;
+            for (int s = 0; s < S; ++s) {
+                const float* uv = V.u + (tr * V.max_segments + s) * 4;
+                const double et = ((double)uv[0] - mg) / mg;
+                const double e =
+                    et * et + ((double)uv[1] * uv[1] + (double)uv[2] * uv[2] + (double)uv[3] * uv[3]) / (tm * tm);
+                total += (double)V.steps[tr * V.max_segments + s] * (double)P.h * (1.0 + (double)P.w_effort * e);
+            }
+            V.cost[tr] = total;
+        }
+    } else {
+        const int w = warp < VAL_COST_WARP ? warp - 1 : warp - 2;
+        int seg0[VAL_PER_WARP], j0[VAL_PER_WARP], done[VAL_PER_WARP], S[VAL_PER_WARP];
+        long long total[VAL_PER_WARP];
+#pragma unroll
+        for (int k = 0; k < VAL_PER_WARP; ++k) {
+            const int i = w + k * VAL_CHECK_WARPS;
+            seg0[k] = j0[k] = 0;
+            total[k] = s_total[i];
+            done[k] = total[k] > 0 ? 0 : 1;
+            S[k] = done[k] ? 0 : V.n_seg[base + i];
+        }
+        for (int c = -1;; ++c) {
+            // c >= 0: the verdicts all warps see for chunk c (see below)
+            if (c >= 0) {
+                const bool all = s_done[c & 1][lane] != 0;
+                if (__all_sync(0xFFFFFFFFu, all)) break;
+            }
+#pragma unroll
+            for (int k = 0; k < VAL_PER_WARP; ++k) {
+                const int i = w + k * VAL_CHECK_WARPS;
+                // the controls of chunk c + 1
+                const long long ahead = total[k] - 32ll * (c + 1);
+                if (!done[k] && ahead > 0)
+                    feed_steps(V, base + i, S[k], seg0[k], j0[k], (int)(ahead < 32 ? ahead : 32),
+                               segment_steps(V, base + i, S[k], seg0[k] + lane), su + ((c + 1) & 1) * 32 * row + i,
+                               sseg + ((c + 1) & 1) * 32 * row + i, row);
+                // the states of chunk c - 1
+                const long long back = total[k] - 32ll * (c - 1);
+                if (c > 0 && !done[k]) {
+                    const int n = (int)(back < 32 ? back : 32);
+                    const float* o = sx + (((c - 1) & 1) * 12 * 32 + lane) * row + i;
+                    float x[12];
+#pragma unroll
+                    for (int d = 0; d < 12; ++d) x[d] = o[d * 32 * row];
+                    bool bad = false;
+                    if (lane < n)
+                        bad = !bounds_ok<12>(P, x) ||
+                              (V.n_obs > 0 && in_a_box<SMEM_BOXES>(P, V, s_box, G, x[0], x[1], x[2]));
+                    const uint32_t b = __ballot_sync(0xFFFFFFFFu, bad);
+                    if (b) {
+                        done[k] = 2;
+                        if (lane == __ffs(b) - 1) {  // the first state that is not valid
+                            V.valid[base + i] = 0;
+                            if (V.x_end)
+#pragma unroll
+                                for (int d = 0; d < 12; ++d) V.x_end[(base + i) * 12 + d] = x[d];
+                        }
+                    } else if (back <= 32) {
+                        done[k] = 1;
+                    }
+                }
+                // read by everyone in the next round; the other buffer is
+                // still being read in this one
+                if (lane == 0) s_done[(c + 1) & 1][i] = done[k];
+            }
+            validate_barrier();
+        }
     }
 }
 
@@ -202,12 +440,23 @@ extern "C" kpx_status kpx_refine_validate(const kpx_dynamics* dyn, const kpx_wor
     V.valid = valid;
     V.cost = cost_out;
     V.x_end = x_end;
-    const size_t smem = (size_t)6 * n_obstacles * sizeof(float);
+    // trajectories per block: as few as one block per SM needs, at most 32; the
+    // boxes in shared memory where they fit beside them
+    const int sms = device_sms();
+    int per_block = (count + sms - 1) / sms;
+    if (per_block > 32) per_block = 32;
+    const int row = per_block | 1;
+    const size_t boxes = (size_t)8 * n_obstacles * sizeof(float);
+    size_t smem = (size_t)VAL_ROW_BYTES * row + VAL_GRID_BYTES;
+    const bool smem_boxes = smem + boxes <= 226 * 1024;
+    if (smem_boxes) smem += boxes;
+    const auto kernel = P.iso_inertia ? (smem_boxes ? k_refine_validate<true, true> : k_refine_validate<true, false>)
+                                      : (smem_boxes ? k_refine_validate<false, true> : k_refine_validate<false, false>);
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_refine_validate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return KPX_E_CUDA;
-    k_refine_validate<<<(count + VAL_WARPS - 1) / VAL_WARPS, VAL_WARPS * 32, smem,
-                        reinterpret_cast<cudaStream_t>(cuda_stream)>>>(P, V);
+    kernel<<<(count + per_block - 1) / per_block, VAL_WARPS * 32, smem, reinterpret_cast<cudaStream_t>(cuda_stream)>>>(
+        P, V, per_block, row);
     return cudaGetLastError() == cudaSuccess ? KPX_OK : KPX_E_CUDA;
 }
 

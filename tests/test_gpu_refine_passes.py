@@ -98,3 +98,31 @@ def test_trajectory_over_the_step_limit():
             assert torch.isnan(J[i]) and not g[i].any()
         else:
             assert J[i] == J0[i] and torch.equal(g[i], g0[i])
+
+
+@pytest.mark.parametrize("count,steps,n_boxes,repeat,aniso", [
+    (1, (1, 3), 0, 1, False), (2, (31, 33), 1, 1, False), (33, (0, 40), 40, 1, True), (153, (5, 9), 300, 1, False),
+    (64, (10, 20), 40, 90, False), (152 * 32 + 5, (3, 12), 60, 1, False),
+])
+def test_validation_batch_equals_its_trajectories_alone(count, steps, n_boxes, repeat, aniso):
+    """Re-validation: a batch against its trajectories alone (exactly) and the
+    FP64 oracle away from boundaries; repeat: the boxes listed many times over
+    and five that fill the workspace's far half, so that the block's grid does
+    not hold them."""
+    prob, x0, u, k, n_seg, obs = _inputs(count, 9, steps, n_boxes, count, aniso)
+    if repeat > 1:
+        obs = np.concatenate([obs, np.tile(np.float32([0.7, 0, 0, 1, 1, 1]), (5, 1))])
+    prob = prob.replace(goal_c=[0.25, 0.5, 0.5], goal_r=0.2)
+    valid, cost, xe = refine.validate(refine.Batch(prob, x0, u, k, n_seg, obstacles=np.tile(obs, (repeat, 1))))
+    agree = 0
+    for i in sorted({0, 1 % count, 31 % count, 32 % count, count // 2, count - 1}):
+        part = slice(i, i + 1)
+        vi, ci, xi = refine.validate(refine.Batch(prob, x0[part], u[part], k[part], n_seg[part], obstacles=obs))
+        assert torch.equal(valid[part], vi) and torch.equal(cost[part], ci) and torch.equal(xe[part], xi), i
+        n = int(n_seg[i])
+        r = oracle.validate_controls(prob.replace(obstacles=obs), x0[i].astype(np.float64), u[i, :n], k[i, :n])
+        assert abs(float(cost[i]) - r["cost"]) <= 1e-12 * max(r["cost"], 1.0)
+        if abs(r["min_clearance"]) >= 1e-4 and abs(r["goal_dist"] - prob.goal_r) >= 1e-4:
+            assert bool(valid[i]) == r["valid"], i
+            agree += 1
+    assert agree >= 1
