@@ -63,8 +63,7 @@ __global__ void __launch_bounds__(1024) k_b_begin(BatchParams BP) {
         return P.hdr->active && P.slot_order ? (P.hdr->n_slots + ORDER_CHUNK - 1) / ORDER_CHUNK : (int64_t)0;
     });
     block_prefix(BP.B, BP.scan_prefix, [&](int p) {
-        const int64_t words = (BP.Ps[p].hdr->n_slots + 31) / 32;
-        return (words + WIN_TILE_WORDS - 1) / WIN_TILE_WORDS;
+        return scan_tiles((BP.Ps[p].hdr->n_slots + 31) / 32, WIN_WORDS_PER_THREAD);
     });
     if (threadIdx.x == 0) {
         for (int c = 0; c < 6; ++c) BP.bh->prop_ticket[c] = 0ull;
@@ -150,7 +149,8 @@ __global__ void __launch_bounds__(WIN_THREADS) k_b_scan(BatchParams BP) {
         const DevParams& P = BP.Ps[p];
         kpx_device_header* H = P.hdr;
         const int64_t n_tiles = BP.scan_prefix[p + 1] - BP.scan_prefix[p];
-        scan_tile(P, H, (uint32_t)(t - BP.scan_prefix[p]), n_tiles, (H->n_slots + 31) / 32, s_warp, s_prefix);
+        scan_tile(P, H, (uint32_t)(t - BP.scan_prefix[p]), n_tiles, (H->n_slots + 31) / 32, WIN_WORDS_PER_THREAD, s_warp,
+                  s_prefix);
     }
 }
 

@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
     kpx_device_header* H = P.hdr;
     if (!H->active) return;
     const int64_t live_words = (H->n_slots + 31) / 32;
-    const int64_t n_tiles = (live_words + WIN_TILE_WORDS - 1) / WIN_TILE_WORDS;
+    const int per = scan_words_per_thread(P, live_words);
+    const int64_t n_tiles = scan_tiles(live_words, per);
     if ((int64_t)blockIdx.x >= n_tiles) return;  // the other blocks take every tile
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(&H->win_ticket, 1u);
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
         const uint32_t tile = s_tile;
         __syncthreads();
         if ((int64_t)tile >= n_tiles) return;
-        scan_tile(P, H, tile, n_tiles, live_words, s_warp, s_prefix);
+        scan_tile(P, H, tile, n_tiles, live_words, per, s_warp, s_prefix);
     }
 }
 
@@ -558,7 +559,7 @@ __global__ void k_wait_timeout(DevParams P, uint64_t* tiles) {
 cudaError_t launch_wait_timeout(const DevParams& P, cudaStream_t s) {
     uint64_t* tiles = P.n_win_tiles >= 2 ? P.win_tiles : (P.n_prune_tiles >= 2 ? P.prune_tiles : nullptr);
     if (!tiles) return cudaErrorInvalidValue;
-    k_wait_timeout<<<1, 1, 0, s>>>(P, tiles);
+    k_wait_timeout<<<1, 32, 0, s>>>(P, tiles);
     return cudaGetLastError();
 }
 

@@ -48,36 +48,42 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T& total, T* s_warp) {
 // an inclusive prefix.  Tile ids come from an atomic ticket, so every
 // predecessor of a waiting tile is already running.  Status word:
 // epoch (30 bits) << 34 | flag (1 aggregate, 2 prefix) << 32 | value.
+// Called by a whole warp: lane l looks at the l-th predecessor, so a tile 32
+// places behind a prefix costs one round trip to L2, not 32 dependent ones.
 // The wait is bounded: after LOOKBACK_POLL_LIMIT polls the kernel records
 // KPX_E_TIMEOUT and continues with the partial prefix.
 __device__ __forceinline__ uint32_t lookback(uint64_t* tiles, uint32_t tile, uint32_t agg, uint32_t epoch,
                                              kpx_device_header* H) {
+    const int lane = threadIdx.x & 31;
     const uint64_t E = (uint64_t)(epoch & 0x3FFFFFFFu);
-    if (tile == 0) {
-        st_relaxed_u64(&tiles[0], (E << 34) | (2ull << 32) | agg);
-        return 0u;
-    }
-    st_relaxed_u64(&tiles[tile], (E << 34) | (1ull << 32) | agg);
+    if (lane == 0) st_relaxed_u64(&tiles[tile], (E << 34) | ((tile == 0 ? 2ull : 1ull) << 32) | agg);
+    if (tile == 0) return 0u;
     uint32_t excl = 0u;
-    int t = (int)tile - 1;
     uint32_t polls = 0;
-    while (t >= 0) {
-        const uint64_t w = ld_relaxed_u64(&tiles[t]);
-        const uint32_t flag = (uint32_t)(w >> 32) & 3u;
-        if ((w >> 34) == E && flag != 0u) {
-            excl += (uint32_t)w;
-            if (flag == 2u) break;
-            --t;
+    for (int t0 = (int)tile - 1; t0 >= 0;) {
+        const int t = t0 - lane;  // before tile 0: a prefix of nothing
+        const uint64_t w = t >= 0 ? ld_relaxed_u64(&tiles[t]) : 0ull;
+        const uint32_t flag = t >= 0 ? ((w >> 34) == E ? (uint32_t)(w >> 32) & 3u : 0u) : 2u;
+        const uint32_t ready = __ballot_sync(FULL, flag != 0u);
+        const uint32_t prefix = __ballot_sync(FULL, flag == 2u);
+        // the nearest predecessors up to the first prefix, or all 32
+        const uint32_t need = prefix ? (prefix ^ (prefix - 1u)) : FULL;
+        if ((ready & need) == need) {
+            excl += __reduce_add_sync(FULL, (need >> lane) & 1u ? (uint32_t)w : 0u);
+            if (prefix) break;
+            t0 -= 32;
         } else {
             if (++polls > LOOKBACK_POLL_LIMIT) {
-                set_status(H, KPX_E_TIMEOUT);
-                H->err_info[0] = 0x10000u | tile;
+                if (lane == 0) {
+                    set_status(H, KPX_E_TIMEOUT);
+                    H->err_info[0] = 0x10000u | tile;
+                }
                 break;
             }
             __nanosleep(32);
         }
     }
-    st_relaxed_u64(&tiles[tile], (E << 34) | (2ull << 32) | (excl + agg));
+    if (lane == 0) st_relaxed_u64(&tiles[tile], (E << 34) | (2ull << 32) | (excl + agg));
     return excl;
 }
 
@@ -589,28 +595,48 @@ __device__ __forceinline__ void mark_region(const DevParams& P, int r) {
 // order -> win_slot[rank]; clears the words.  The problem's last tile writes
 // its winner count.
 // ---------------------------------------------------------------------------
+// Words a thread takes: as few as the problem's tile words allow, so that an
+// iteration of a few hundred thousand slots spreads over all of its blocks
+// (11 tiles instead of 2 at 85,000 slots: 5.2 -> 4.3 us; 41 instead of 5 at
+// 325,000: 9.1 -> 5.2 us).  A batch keeps whole tiles: its problems fill the
+// blocks, and more tiles only cost it (12.5 -> 18.7 us for 48 problems).
+__device__ __forceinline__ int scan_words_per_thread(const DevParams& P, int64_t live_words) {
+    int n = 1;
+    while (n < WIN_WORDS_PER_THREAD && live_words > (int64_t)P.n_win_tiles * (WIN_THREADS * n)) n *= 2;
+    return n;
+}
+
+// per: words a thread (1, 2, 4 or WIN_WORDS_PER_THREAD)
+__device__ __forceinline__ int64_t scan_tiles(int64_t live_words, int per) {
+    return (live_words + WIN_THREADS * per - 1) / (WIN_THREADS * per);
+}
+
 __device__ __forceinline__ void scan_tile(const DevParams& P, kpx_device_header* H, uint32_t tile, int64_t n_tiles,
-                                          int64_t live_words, uint32_t* s_warp, uint32_t& s_prefix) {
-    const int64_t w0 = (int64_t)tile * WIN_TILE_WORDS + (int64_t)threadIdx.x * WIN_WORDS_PER_THREAD;
+                                          int64_t live_words, int per, uint32_t* s_warp, uint32_t& s_prefix) {
+    const int64_t w0 = ((int64_t)tile * WIN_THREADS + threadIdx.x) * per;
     static_assert(WIN_WORDS_PER_THREAD == 8, "two 16-byte loads a thread");
     uint32_t w[WIN_WORDS_PER_THREAD];
     uint32_t cnt = 0;
-    if (w0 + WIN_WORDS_PER_THREAD <= live_words) {  // w0 is a multiple of 8 words: 32-byte aligned
+    if (per == WIN_WORDS_PER_THREAD && w0 + WIN_WORDS_PER_THREAD <= live_words) {  // 32-byte aligned
         const uint4 a = *reinterpret_cast<const uint4*>(P.win_mask + w0);
         const uint4 b = *reinterpret_cast<const uint4*>(P.win_mask + w0 + 4);
         w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
         w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
     } else {
 #pragma unroll
-        for (int i = 0; i < WIN_WORDS_PER_THREAD; ++i) w[i] = (w0 + i < live_words) ? P.win_mask[w0 + i] : 0u;
+        for (int i = 0; i < WIN_WORDS_PER_THREAD; ++i)
+            w[i] = (i < per && w0 + i < live_words) ? P.win_mask[w0 + i] : 0u;
     }
 #pragma unroll
     for (int i = 0; i < WIN_WORDS_PER_THREAD; ++i) cnt += __popc(w[i]);
     uint32_t agg;
     const uint32_t excl = block_exclusive_scan<WIN_THREADS>(cnt, agg, s_warp);
-    if (threadIdx.x == 0) {
-        s_prefix = lookback(P.win_tiles, tile, agg, (uint32_t)H->epoch, H);
-        if ((int64_t)tile == n_tiles - 1) H->n_win = (int32_t)(s_prefix + agg);
+    if (threadIdx.x < 32) {
+        const uint32_t prefix = lookback(P.win_tiles, tile, agg, (uint32_t)H->epoch, H);
+        if (threadIdx.x == 0) {
+            s_prefix = prefix;
+            if ((int64_t)tile == n_tiles - 1) H->n_win = (int32_t)(prefix + agg);
+        }
     }
     __syncthreads();
     uint32_t rank = s_prefix + excl;
@@ -924,9 +950,10 @@ __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header
         const uint32_t agg = __shfl_sync(FULL, x, 31);
         __syncwarp();
         if (lane < PRUNE_ROUND_WARPS) s_counts[lane] = x - v;
+        const uint32_t prefix = lookback(P.prune_tiles, tile, agg, epoch, H);
         if (lane == 0) {
-            s_prefix = lookback(P.prune_tiles, tile, agg, epoch, H);
-            if ((int)tile == n_tiles - 1) H->count_A_next = (int32_t)(s_prefix + agg);
+            s_prefix = prefix;
+            if ((int)tile == n_tiles - 1) H->count_A_next = (int32_t)(prefix + agg);
         }
     }
     __syncthreads();
