@@ -262,10 +262,11 @@ kpx_status kpx_set_regions(kpx_planner* p, int32_t n_axes, const kpx_region_axis
  * cluster while an iteration has at most one 32-slot chunk per warp of the
  * cluster and the tree at most 32,768 nodes, and leaves the iterations it
  * did not run in graph_pending.  A loop (a WHILE conditional node) then runs
- * the eight phase kernels once per iteration left, counting graph_pending
- * down to 0.  A launch of n iterations thus starts 1 + 8 m kernels, m = the
- * iterations the fused kernel left (the header's fused_iterations counts the
- * ones it ran); without the fused kernel, 7 n. */
+ * seven phase kernels once per iteration left (the last block of the last
+ * two counts it off graph_pending), until that is 0.  A launch of n
+ * iterations thus starts 1 + 7 m kernels, m = the iterations the fused
+ * kernel left (the header's fused_iterations counts the ones it ran);
+ * without the fused kernel, 7 n. */
 kpx_status kpx_graph_info(kpx_planner* p, int32_t* max_iterations_per_launch, int32_t* fused);
 
 /* Waits for the planner's stream and releases the host handle; the device

@@ -342,25 +342,26 @@ constexpr int kLoopIterations = 8;
 constexpr int kLoopIterationsFused = 2;
 
 // One iteration of the phase kernels in the body of the graph's loop: it
-// runs only while iterations are owed, and its last kernel counts it off
-// graph_pending (the body's last iteration sets the loop's handle).
+// runs only while iterations are owed.
 // The kept winners' re-integration (stage) forks onto the side stream after
-// the winner scan and joins before the iteration's end, so that it runs
-// beside append and prune (which need no end state).
+// the winner scan and joins after prune, so that it runs beside append and
+// prune (which need no end state).  The last block of the two to finish ends
+// the iteration and counts it off graph_pending (the body's last iteration
+// sets the loop's handle).
 cudaError_t enqueue_loop_iteration(const DevParams& P, cudaGraphConditionalHandle h, bool last, cudaStream_t s,
                                    const SideBranch& side) {
+    const LoopEnd end = loop_end(P, h, last);
     cudaError_t e = launch_begin(P, s, true);
     if (e == cudaSuccess) e = launch_propagate(P, nullptr, s);
     if (e == cudaSuccess) e = launch_mark(P, s);
     if (e == cudaSuccess) e = launch_scan(P, s);
     if (e == cudaSuccess) e = cudaEventRecord(side.fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side.stream, side.fork, 0);
-    if (e == cudaSuccess) e = launch_stage(P, side.stream);
+    if (e == cudaSuccess) e = launch_stage(P, side.stream, &end);
     if (e == cudaSuccess) e = cudaEventRecord(side.join, side.stream);
     if (e == cudaSuccess) e = launch_append(P, s);
-    if (e == cudaSuccess) e = launch_prune(P, s);
+    if (e == cudaSuccess) e = launch_prune(P, s, &end);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, side.join, 0);
-    if (e == cudaSuccess) e = launch_end_loop(P, h, last, s);
     return e;
 }
 

@@ -266,13 +266,17 @@ cudaError_t launch_scan(const DevParams& P, cudaStream_t s);
 // UpdateTree in two halves (kpx_phases.cuh): append (rows, keys, owners,
 // capacity rule) and stage (the kept winners' end states and the goal test)
 cudaError_t launch_append(const DevParams& P, cudaStream_t s);
-cudaError_t launch_stage(const DevParams& P, cudaStream_t s);
-cudaError_t launch_prune(const DevParams& P, cudaStream_t s);
+// In the loop body of a planner's graph (end != null) the last block of stage
+// and prune to finish also ends the iteration.
+struct LoopEnd {
+    cudaGraphConditionalHandle handle;
+    int32_t mode;   // 0: no end here; 1: an iteration of the body; 2: its last one (sets the handle)
+    int32_t stage_blocks, prune_blocks;  // the two launches' grids
+};
+cudaError_t launch_stage(const DevParams& P, cudaStream_t s, const LoopEnd* end = nullptr);
+cudaError_t launch_prune(const DevParams& P, cudaStream_t s, const LoopEnd* end = nullptr);
+LoopEnd loop_end(const DevParams& P, cudaGraphConditionalHandle h, bool last);
 cudaError_t launch_end(const DevParams& P, cudaStream_t s);
-// the end of an iteration in the loop body of a planner's graph: counts the
-// iteration off graph_pending; the body's last sets the loop's handle (1: run
-// again)
-cudaError_t launch_end_loop(const DevParams& P, cudaGraphConditionalHandle h, bool last, cudaStream_t s);
 cudaError_t launch_path(const DevParams& P, cudaStream_t s);
 // one bounded look-back wait that nothing releases (tests): records KPX_E_TIMEOUT
 cudaError_t launch_wait_timeout(const DevParams& P, cudaStream_t s);

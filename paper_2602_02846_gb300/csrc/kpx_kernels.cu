@@ -35,6 +35,20 @@ namespace kpx {
 
 namespace {
 
+// The phase kernels are launched with programmatic stream serialization
+// (launch_pdl): a kernel's blocks may be set up while the one before it in the
+// stream drains, and wait here, at the very top of every one of them, until it
+// has completed and its writes are visible; a kernel so completes only after
+// all the ones before it.  Without the launch attribute the wait is empty.
+// (No early launch_dependents: the next kernels' waiting blocks then sat on
+// the SMs and the dependent chain slowed down, 4.09 -> 4.29 ms among 30
+// columns.)  Against plain launches and a kernel of its own for the
+// iteration's end: static_di 1341 -> 1151 us, plan_di_room 646 -> 625,
+// plan_dubins_open -2.6 %.
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // init / reset: Alg. 1 initialisation.
 // ---------------------------------------------------------------------------
@@ -171,6 +185,7 @@ __global__ void __launch_bounds__(1024) k_grid_scan(DevParams P) {
 // from counters begin_counters leaves alone (|V_A|, the iteration, the V_A
 // buffer), exactly as begin_counters derives them.
 __global__ void k_begin(DevParams P, int loop) {
+    pdl_enter();
     kpx_device_header* H = P.hdr;
     const bool allowed = !loop || H->graph_pending > 0;
     const bool snap = begin_needs_snapshot(P, H, allowed);  // reads counters begin_counters leaves alone
@@ -215,6 +230,7 @@ struct PropOccupancy {
 template <int DYN, int INTEG, bool SYM>
 __global__ void __launch_bounds__(PROP_THREADS, PropOccupancy<DYN>::blocks)
     k_propagate(DevParams P, kpx_debug_records rec, int rec_on) {
+    pdl_enter();
     kpx_device_header* H = P.hdr;
     if (!H->active) return;
     const int64_t n_slots = H->n_slots;
@@ -239,11 +255,13 @@ __global__ void __launch_bounds__(PROP_THREADS, PropOccupancy<DYN>::blocks)
 }
 
 __global__ void k_mark(DevParams P) {
+    pdl_enter();
     if (!P.hdr->active) return;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < P.R; r += gridDim.x * blockDim.x) mark_region(P, r);
 }
 
 __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
+    pdl_enter();
     __shared__ uint32_t s_tile, s_prefix;
     __shared__ uint32_t s_warp[WIN_THREADS / 32];
     kpx_device_header* H = P.hdr;
@@ -264,6 +282,7 @@ __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
 
 template <int DYN, int INTEG>
 __global__ void __launch_bounds__(128) k_append(DevParams P) {
+    pdl_enter();
     kpx_device_header* H = P.hdr;
     if (!H->active) return;
     const int W = H->n_win;
@@ -273,6 +292,10 @@ __global__ void __launch_bounds__(128) k_append(DevParams P) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         H->n_kept = kept;
         if (W > kept) set_status(H, KPX_TREE_FULL);
+        // the winner scan is over: its ticket word holds prune's tile count,
+        // which a prune block must not derive from the tree size (a block
+        // that starts late may find the iteration already ended)
+        H->win_ticket = (uint32_t)((n_old + kept + PRUNE_TILE - 1) / PRUNE_TILE);
     }
     const int lam = H->lambda;
     const uint32_t iter = (uint32_t)H->iter;
@@ -281,35 +304,84 @@ __global__ void __launch_bounds__(128) k_append(DevParams P) {
         append_meta<DYN, INTEG>(P, H, w, kept, n_old, lam, iter, va);
 }
 
+// The end of an iteration in the loop body of a planner's graph, by the last
+// working block of stage and prune to finish (no kernel of its own: 2.3 us and
+// a kernel boundary per iteration).  Called by one block; `blocks`: the working
+// blocks of both launches, which each caller derives from the iteration's
+// winners and tiles before it reports.  The count is kept in graph_ctl, which
+// is 0 between iterations.
+// An iteration that ran (graph_pending > 0, as k_begin saw it) ends and is
+// counted off; once the problem has stopped (tree full, an error, its
+// iteration limit) the iterations still owed would be no-ops and are
+// dropped.  The body's last iteration lets the loop run again while
+// iterations are owed.  graph_pending only falls, so the loop ends.
+__device__ __forceinline__ void finish_block(const DevParams& P, const LoopEnd& E, int blocks) {
+    if (E.mode == 0) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    kpx_device_header* H = P.hdr;
+    __threadfence();
+    if (atomicAdd(&H->graph_ctl, 1) != blocks - 1) return;
+    __threadfence();
+    H->graph_ctl = 0;
+    if (H->graph_pending > 0) {
+        end_counters(P, H);
+        H->graph_pending = problem_runs(P, H) ? H->graph_pending - 1 : 0;
+    }
+    if (E.mode == 2) cudaGraphSetConditional(E.handle, H->graph_pending > 0 ? 1u : 0u);
+}
+
+// The blocks of a launch that have work, at least one.
+__device__ __forceinline__ int working_blocks(int grid, int64_t work) {
+    return (int)(work < 1 ? 1 : (work < grid ? work : grid));
+}
+
+constexpr int STAGE_THREADS = 128;
+
 // The kept winners' end states (one thread per winner, re-materialised) and
 // the solution update; in the planner's graphs beside append and prune.
 template <int DYN, int INTEG>
-__global__ void __launch_bounds__(128) k_stage(DevParams P) {
+__global__ void __launch_bounds__(STAGE_THREADS) k_stage(DevParams P, LoopEnd E) {
+    pdl_enter();
     kpx_device_header* H = P.hdr;
-    if (!H->active) return;
+    if (!H->active) {
+        if (blockIdx.x == 0) finish_block(P, E, 2);
+        return;
+    }
     const int W = H->n_win;
     const int n_old = H->n_nodes;  // end_counters advances it only after both halves
     const int room = P.N - n_old;
     const int kept = W < room ? W : room;
+    // A block that starts after the iteration's end (it has no work, so the end
+    // did not wait for it) sees less room and so still no work.
+    const int working = working_blocks((int)gridDim.x, (kept + STAGE_THREADS - 1) / STAGE_THREADS);
+    if ((int)blockIdx.x >= working) return;
     const int lam = H->lambda;
     const uint32_t iter = (uint32_t)H->iter;
     const int32_t* va = va_current(P, H);
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < kept; w += gridDim.x * blockDim.x)
+    const int tiles = (n_old + kept + PRUNE_TILE - 1) / PRUNE_TILE;
+    for (int w = blockIdx.x * STAGE_THREADS + threadIdx.x; w < kept; w += gridDim.x * STAGE_THREADS)
         stage_winner<DYN, INTEG>(P, H, w, n_old, lam, iter, va);
+    finish_block(P, E, working + working_blocks(E.prune_blocks, tiles));
 }
 
-__global__ void __launch_bounds__(PRUNE_THREADS, 8) k_prune(DevParams P) {
+__global__ void __launch_bounds__(PRUNE_THREADS, 8) k_prune(DevParams P, LoopEnd E) {
+    pdl_enter();
     __shared__ uint32_t s_tile, s_prefix;
     __shared__ int32_t s_parent[PRUNE_TILE];
     __shared__ uint8_t s_set[PRUNE_TILE];
     __shared__ uint8_t s_icount[PRUNE_TILE];
     __shared__ uint32_t s_counts[PRUNE_ROUND_WARPS];
     kpx_device_header* H = P.hdr;
-    if (!H->active) return;
-    const int n_old = H->n_nodes;
-    const int total = n_old + H->n_kept;
-    const int n_tiles = (total + PRUNE_TILE - 1) / PRUNE_TILE;
+    if (!H->active) {
+        if (blockIdx.x == 0) finish_block(P, E, 2);
+        return;
+    }
+    const int n_tiles = (int)H->win_ticket;  // append's
     if ((int)blockIdx.x >= n_tiles) return;  // the other blocks take every tile
+    const int n_old = H->n_nodes;
+    const int kept = H->n_kept;
+    const int total = n_old + kept;
     const uint32_t epoch = (uint32_t)H->epoch;
     int32_t* va_next = va_following(P, H);
     int cA = 0, cI = 0, cT = 0;
@@ -323,23 +395,13 @@ __global__ void __launch_bounds__(PRUNE_THREADS, 8) k_prune(DevParams P) {
                    cA, cI, cT);
     }
     flush_prune_counters(H, cA, cI, cT);
+    finish_block(P, E, working_blocks((int)gridDim.x, n_tiles) +
+                           working_blocks(E.stage_blocks, (kept + STAGE_THREADS - 1) / STAGE_THREADS));
 }
 
-__global__ void k_end(DevParams P) { end_counters(P, P.hdr); }
-
-// The end of an iteration in the loop body of a planner's graph: an
-// iteration that ran (graph_pending > 0, as k_begin saw it) ends and is
-// counted off; once the problem has stopped (tree full, an error, its
-// iteration limit) the iterations still owed would be no-ops and are
-// dropped.  The body's last iteration lets the loop run again while
-// iterations are owed.  graph_pending only falls, so the loop ends.
-__global__ void k_end_loop(DevParams P, cudaGraphConditionalHandle h, int last) {
-    kpx_device_header* H = P.hdr;
-    if (H->graph_pending > 0) {
-        end_counters(P, H);
-        H->graph_pending = problem_runs(P, H) ? H->graph_pending - 1 : 0;
-    }
-    if (last) cudaGraphSetConditional(h, H->graph_pending > 0 ? 1u : 0u);
+__global__ void k_end(DevParams P) {
+    pdl_enter();
+    end_counters(P, P.hdr);
 }
 
 // ---------------------------------------------------------------------------
@@ -413,6 +475,27 @@ __global__ void k_remap_mark(DevParams P) {
     }
 }
 
+// pdl false: an ordinary launch (a kernel that joins two branches of a graph,
+// or starts one)
+template <typename... K, typename... A>
+cudaError_t launch_kernel(bool pdl, void (*k)(K...), int grid, int block, cudaStream_t s, A... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, K(a)...);
+}
+
+template <typename... K, typename... A>
+cudaError_t launch_pdl(void (*k)(K...), int grid, int block, cudaStream_t s, A... a) {
+    return launch_kernel(true, k, grid, block, s, a...);
+}
+
 int sm_count() {
     static int cached[64] = {};
     int dev = 0;
@@ -462,23 +545,24 @@ cudaError_t launch_propagate_t(const DevParams& P, const kpx_debug_records* rec,
         r = *rec;
         on = 1;
     }
-    if (P.sym_bounds)
-        k_propagate<DYN, INTEG, true><<<grid, PROP_THREADS, 0, s>>>(P, r, on);
-    else
-        k_propagate<DYN, INTEG, false><<<grid, PROP_THREADS, 0, s>>>(P, r, on);
-    return cudaGetLastError();
+    return launch_pdl(P.sym_bounds ? k_propagate<DYN, INTEG, true> : k_propagate<DYN, INTEG, false>, grid, PROP_THREADS,
+                      s, P, r, on);
 }
 
 template <int DYN, int INTEG>
 cudaError_t launch_append_t(const DevParams& P, cudaStream_t s) {
-    k_append<DYN, INTEG><<<persistent_blocks((P.R + 127) / 128, 4), 128, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(k_append<DYN, INTEG>, persistent_blocks((P.R + 127) / 128, 4), 128, s, P);
 }
 
+int stage_blocks(const DevParams& P) { return persistent_blocks((P.R + STAGE_THREADS - 1) / STAGE_THREADS, 4); }
+
+// a tile's time is its deepest ancestor walk: as many tiles in flight as fit
+// (32 registers and 6 KB of shared memory a block: 8 blocks per SM)
+int prune_blocks(const DevParams& P) { return persistent_blocks(P.n_prune_tiles, 8); }
+
 template <int DYN, int INTEG>
-cudaError_t launch_stage_t(const DevParams& P, cudaStream_t s) {
-    k_stage<DYN, INTEG><<<persistent_blocks((P.R + 127) / 128, 4), 128, 0, s>>>(P);
-    return cudaGetLastError();
+cudaError_t launch_stage_t(const DevParams& P, cudaStream_t s, const LoopEnd& end) {
+    return launch_kernel(end.mode == 0, k_stage<DYN, INTEG>, stage_blocks(P), STAGE_THREADS, s, P, end);
 }
 
 }  // namespace
@@ -515,8 +599,7 @@ cudaError_t launch_begin(const DevParams& P, cudaStream_t s, bool loop) {
         if (order_blocks > work) work = order_blocks;
         per_sm = 6;
     }
-    k_begin<<<persistent_blocks(work, per_sm), 256, 0, s>>>(P, loop ? 1 : 0);
-    return cudaGetLastError();
+    return launch_kernel(!loop, k_begin, persistent_blocks(work, per_sm), 256, s, P, loop ? 1 : 0);
 }
 
 cudaError_t launch_propagate(const DevParams& P, const kpx_debug_records* rec, cudaStream_t s) {
@@ -524,25 +607,27 @@ cudaError_t launch_propagate(const DevParams& P, const kpx_debug_records* rec, c
 }
 
 cudaError_t launch_mark(const DevParams& P, cudaStream_t s) {
-    k_mark<<<persistent_blocks((P.R + 255) / 256, 8), 256, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(k_mark, persistent_blocks((P.R + 255) / 256, 8), 256, s, P);
 }
 
 // every tile of a large iteration in flight at once (31 registers: 8 blocks per SM)
 cudaError_t launch_scan(const DevParams& P, cudaStream_t s) {
-    k_scan<<<persistent_blocks(P.n_win_tiles, 8), WIN_THREADS, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(k_scan, persistent_blocks(P.n_win_tiles, 8), WIN_THREADS, s, P);
 }
 
 cudaError_t launch_append(const DevParams& P, cudaStream_t s) { KPX_DISPATCH(launch_append_t, P, s); }
 
-cudaError_t launch_stage(const DevParams& P, cudaStream_t s) { KPX_DISPATCH(launch_stage_t, P, s); }
+LoopEnd loop_end(const DevParams& P, cudaGraphConditionalHandle h, bool last) {
+    return LoopEnd{h, last ? 2 : 1, stage_blocks(P), prune_blocks(P)};
+}
 
-cudaError_t launch_prune(const DevParams& P, cudaStream_t s) {
-    // a tile's time is its deepest ancestor walk: as many tiles in flight as fit
-    // (32 registers and 6 KB of shared memory a block: 8 blocks per SM)
-    k_prune<<<persistent_blocks(P.n_prune_tiles, 8), PRUNE_THREADS, 0, s>>>(P);
-    return cudaGetLastError();
+cudaError_t launch_stage(const DevParams& P, cudaStream_t s, const LoopEnd* end) {
+    const LoopEnd e = end ? *end : LoopEnd{};
+    KPX_DISPATCH(launch_stage_t, P, s, e);
+}
+
+cudaError_t launch_prune(const DevParams& P, cudaStream_t s, const LoopEnd* end) {
+    return launch_pdl(k_prune, prune_blocks(P), PRUNE_THREADS, s, P, end ? *end : LoopEnd{});
 }
 
 // A look-back wait that nothing will release: tile 1 of `tiles` waits on
@@ -563,14 +648,8 @@ cudaError_t launch_wait_timeout(const DevParams& P, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_end_loop(const DevParams& P, cudaGraphConditionalHandle h, bool last, cudaStream_t s) {
-    k_end_loop<<<1, 1, 0, s>>>(P, h, last ? 1 : 0);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_end(const DevParams& P, cudaStream_t s) {
-    k_end<<<1, 1, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(k_end, 1, 1, s, P);
 }
 
 cudaError_t launch_remap_regions(const DevParams& P, cudaStream_t s) {
