@@ -169,7 +169,7 @@ Layout make_layout(const kpx_dynamics* dyn, const kpx_config* cfg, int32_t n_obs
     };
     L.hdr = seg(sizeof(kpx_device_header));
     L.obs = seg((size_t)(n_obs > 0 ? n_obs : 1) * 2 * sizeof(float4));
-    L.box_cells = seg((size_t)(n_obs > 0 ? n_obs : 1) * 6 * sizeof(int32_t));
+    seg((size_t)(n_obs > 0 ? n_obs : 1) * 6 * sizeof(int32_t));  // unused: keeps the offsets of saved snapshots
     L.cell_start = seg((size_t)(GRID_MAX_CELLS + 1) * sizeof(int32_t));
     L.cell_pair = seg((size_t)GRID_MAX_CELLS * sizeof(int2));
     L.cell_box = seg((size_t)grid_entry_budget(n_obs) * 2 * sizeof(float4));
@@ -284,7 +284,6 @@ void bind_pointers(kpx_planner* p) {
     DevParams& P = p->P;
     P.hdr = reinterpret_cast<kpx_device_header*>(b + L.hdr);
     P.obs = reinterpret_cast<float4*>(b + L.obs);
-    P.box_cells = reinterpret_cast<int32_t*>(b + L.box_cells);
     P.cell_start = reinterpret_cast<int32_t*>(b + L.cell_start);
     P.cell_pair = reinterpret_cast<int2*>(b + L.cell_pair);
     P.cell_box = reinterpret_cast<float4*>(b + L.cell_box);

@@ -106,7 +106,6 @@ struct DevParams {
     uint64_t* win_tiles;
     uint64_t* prune_tiles;
     float4* obs;          // [2*n_obs]: lo (x,y,z,0), hi (x,y,z,0)
-    int32_t* box_cells;   // [6*n_obs]: per box cell range lo x,y,z, hi x,y,z
     int32_t* cell_start;  // [n_cells + 1]: CSR offsets into cell_box
     int2* cell_pair;      // [n_cells]: (cell_start[c], min(cell_start[c + 1], grid_cap)), one 8-byte load
     float4* cell_box;     // [2*grid_cap]: boxes of each cell, in box order
@@ -136,7 +135,7 @@ __host__ __device__ inline int grid_cell(float c, float lo, float inv, int n) {
 
 // Workspace layout (byte offsets from the workspace base).
 struct Layout {
-    size_t hdr, obs, box_cells, cell_start, cell_pair, cell_box, x, u, K, parent, key, region, set, icount;
+    size_t hdr, obs, cell_start, cell_pair, cell_box, x, u, K, parent, key, region, set, icount;
     size_t region_key, region_snap, region_owner, va0, va1, win_slot, win_mask, win_tiles, prune_tiles, clean,
         slot_region, slot_order, path, traj;
     size_t total;
