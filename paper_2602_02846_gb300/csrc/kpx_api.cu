@@ -1326,13 +1326,17 @@ kpx_status kpx_restore(kpx_planner* p, const void* src) {
 // process exits.  The call synchronises its stream, so it refuses to run
 // while that stream is being captured into a CUDA graph.  Validation and the
 // parameter block are kpx_create's (validate_problem, fill_problem), and the
-// iterations are the phase kernels of enqueue_iteration.
+// iterations are the fused kernel's and the phase kernels' (plain launches: a
+// CUDA graph would be allocated).
 // ===========================================================================
 namespace {
 
 constexpr size_t kStaticScratchBytes = (size_t)KPX_STATIC_SCRATCH_BYTES;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+
+// phase-kernel iterations launched ahead of a look at the planner's state
+constexpr int32_t kStaticIterations = 8;
 
 // Device address of g_static_scratch, looked up once per device with that
 // device current (the host-side symbol is only a stand-in, never a device
@@ -1432,11 +1436,33 @@ extern "C" kpx_status kpx_plan_static(const kpx_dynamics* dyn, const kpx_workspa
     // every array that must start at zero is cleared by the first-time init
     if (e == cudaSuccess) e = launch_init(P, true, pl.stream);
     if (e == cudaSuccess) e = launch_grid_build(P, pl.stream);
-    for (int32_t it = 0; e == cudaSuccess && it < n_iters; ++it) e = enqueue_iteration(P, pl.stream);
-    if (e == cudaSuccess) e = launch_path(P, pl.stream);
+    // whole iterations in the one-cluster kernel while the problem is small
+    // (bit-identical), then the phase kernels for those it leaves.  Their host
+    // loop looks at the planner's state every kStaticIterations: a full tree
+    // makes the rest no-ops, which are not launched then.
     kpx_device_header h;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, P.hdr, sizeof(h), cudaMemcpyDeviceToHost, pl.stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(pl.stream);
+    auto sync_header = [&]() {
+        cudaError_t he = cudaMemcpyAsync(&h, P.hdr, sizeof(h), cudaMemcpyDeviceToHost, pl.stream);
+        return he == cudaSuccess ? cudaStreamSynchronize(pl.stream) : he;
+    };
+    int32_t left = n_iters;
+    if (e == cudaSuccess && left > 0 && !(P.flags & KPX_FLAG_NO_FUSED) && fused_cluster_size(P) > 0 &&
+        launch_fused(P, left, 0, 0, pl.stream) == cudaSuccess) {
+        e = sync_header();
+        left = e == cudaSuccess ? h.graph_pending : 0;
+    }
+    cudaGetLastError();  // an unavailable cluster launch leaves every iteration to the phase kernels
+    while (e == cudaSuccess && left > 0) {
+        const int32_t n = left < kStaticIterations ? left : kStaticIterations;
+        for (int32_t it = 0; e == cudaSuccess && it < n; ++it) e = enqueue_iteration(P, pl.stream);
+        left -= n;
+        if (e == cudaSuccess && left > 0) {
+            e = sync_header();
+            if (e == cudaSuccess && h.status != KPX_OK) left = 0;
+        }
+    }
+    if (e == cudaSuccess) e = launch_path(P, pl.stream);
+    if (e == cudaSuccess) e = sync_header();
     if (e != cudaSuccess) {
         g_create_error = std::string("kpx_plan_static: ") + cudaGetErrorString(e);
         return KPX_E_CUDA;
