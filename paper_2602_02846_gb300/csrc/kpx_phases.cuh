@@ -168,7 +168,10 @@ __device__ __forceinline__ bool begin_needs_snapshot(const DevParams& P, const k
 // propagate order: the slots of each aligned ORDER_CHUNK-slot chunk sorted by
 // an order key, their step count K or the quadcopter's predicted step count
 // (one warp per chunk, a bitonic network over the warp's registers and
-// shuffles).  Only the lane that computes a slot changes, not the slot's
+// shuffles).  Bound: issue (the Philox rounds, then the network): 20.2 -> 16.9
+// us a launch in the quadcopter building with one slot division a lane
+// instead of four, one quotient an axis in the quadcopter's key and two 16-bit
+// values a register in the network.  Only the lane that computes a slot changes, not the slot's
 // result.
 // ---------------------------------------------------------------------------
 // Ascending sort of the 128 values v[e] of all lanes, element i = lane + 32 e.
@@ -201,6 +204,47 @@ __device__ __forceinline__ void warp_sort128(uint32_t (&v)[4]) {
             }
         }
     }
+}
+
+// The same for values below 2^16, two a register: a holds elements e = 0 (low
+// half) and 2, b holds 1 and 3; half the shuffles, and a packed 16-bit minimum
+// or maximum serves both halves.  A descending half is sorted complemented.
+__device__ __forceinline__ void warp_sort128_16(uint32_t& a, uint32_t& b) {
+    const int lane = threadIdx.x & 31;
+    // one stage against the elements j lanes away; desc_b: b runs descending
+    auto stage = [&](int j, bool asc_a, bool asc_b) {
+        const uint32_t oa = __shfl_xor_sync(FULL, a, j), ob = __shfl_xor_sync(FULL, b, j);
+        const bool lower = (lane & j) == 0;
+        a = lower == asc_a ? __vminu2(a, oa) : __vmaxu2(a, oa);
+        b = lower == asc_b ? __vminu2(b, ob) : __vmaxu2(b, ob);
+    };
+    auto between = [&]() {  // elements 0, 1 and 2, 3: a takes the smaller ones
+        const uint32_t lo = __vminu2(a, b), hi = __vmaxu2(a, b);
+        a = lo;
+        b = hi;
+    };
+#pragma unroll
+    for (int k = 2; k <= 16; k <<= 1) {
+        const bool asc = (lane & k) == 0;
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) stage(j, asc, asc);
+    }
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) stage(j, true, false);  // runs of 32: element's bit 0 gives the direction
+    a ^= 0xFFFF0000u;  // runs of 64: elements 2 and 3 descend
+    b ^= 0xFFFF0000u;
+    between();
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) stage(j, true, true);
+    a ^= 0xFFFF0000u;
+    b ^= 0xFFFF0000u;
+    // the whole: first each half against the other
+    const uint32_t sa = __byte_perm(a, a, 0x1032), sb = __byte_perm(b, b, 0x1032);
+    a = __byte_perm(__vminu2(a, sa), __vmaxu2(a, sa), 0x7610);
+    b = __byte_perm(__vminu2(b, sb), __vmaxu2(b, sb), 0x7610);
+    between();
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) stage(j, true, true);
 }
 
 // The sort key of a quadcopter slot: K, or fewer steps when the velocity,
@@ -243,11 +287,16 @@ __device__ __forceinline__ uint32_t quad_order_key(const DevParams& P, const Qua
     float n = (float)K;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        if (dv[i] > 0.0f) n = fminf(n, __fdividef(P.x_hi[6 + i] - q.v[i], dv[i]));
-        if (dv[i] < 0.0f) n = fminf(n, __fdividef(P.x_lo[6 + i] - q.v[i], dv[i]));
+        // the bound the velocity moves to
+        const float room = (dv[i] > 0.0f ? P.x_hi[6 + i] : P.x_lo[6 + i]) - q.v[i];
+        if (dv[i] != 0.0f) n = fminf(n, __fdividef(room, dv[i]));
     }
     return (uint32_t)fmaxf(n, 0.0f);  // <= K < 2^16
 }
+
+// the largest step count whose keys sort as 16-bit values: (510 << 7 | 127) is below
+// a dead slot's 0xFF80
+constexpr int ORDER_KEY16_MAX = 510;
 
 // Chunk c of this iteration's slots: order[c * 128 + p] = offset in the
 // chunk of the slot with the p-th smallest (key, offset), the key being K
@@ -261,30 +310,49 @@ __device__ __forceinline__ void order_chunk(const DevParams& P, const int32_t* v
     uint32_t v[4];
     int j_parent = -1;  // the parent whose part of the quadcopter key qp holds
     QuadOrderParent qp;
+    // the slot's parent rank and sample: one division, then 32 samples on
+    const uint32_t s0 = (uint32_t)(c * ORDER_CHUNK) + (uint32_t)lane;  // < 2^32, as in LaneRollout::start
+    uint32_t j = s0 / (uint32_t)lam;
+    uint32_t s = s0 - j * (uint32_t)lam;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const uint32_t off = (uint32_t)(lane + 32 * e);
+        if (e > 0) {
+            s += 32u;
+            if (s >= (uint32_t)lam) {
+                const uint32_t q = lam >= 32 ? 1u : s / (uint32_t)lam;
+                j += q;
+                s -= q * (uint32_t)lam;
+            }
+        }
         const int64_t slot = c * ORDER_CHUNK + off;
         if (slot < n_slots) {
-            const uint32_t su = (uint32_t)slot;  // < 2^32, as in LaneRollout::start
-            const int j = (int)(su / (uint32_t)lam);
-            const int s = (int)(su - (uint32_t)j * (uint32_t)lam);
             uint32_t key;
+            const int node = va[j];
             if constexpr (M == 4) {
-                if (j != j_parent) {
-                    qp = quad_order_parent(P, va[j]);
-                    j_parent = j;
+                if ((int)j != j_parent) {
+                    qp = quad_order_parent(P, node);
+                    j_parent = (int)j;
                 }
-                key = quad_order_key(P, qp, va[j], iter, (uint32_t)s);
+                key = quad_order_key(P, qp, node, iter, s);
             } else {
-                key = (uint32_t)sample_steps<M>(P, iter, (uint32_t)va[j], (uint32_t)s);
+                key = (uint32_t)sample_steps<M>(P, iter, (uint32_t)node, s);
             }
             v[e] = (key << 7) | off;  // key < 2^16
         } else {
             v[e] = 0xFFFFFF80u | off;
         }
     }
-    warp_sort128(v);
+    if (P.k_max <= ORDER_KEY16_MAX) {  // every live value below 0xFF80: 16 bits hold it, and a dead slot's
+        uint32_t a = __byte_perm(v[0], v[2], 0x5410), b = __byte_perm(v[1], v[3], 0x5410);
+        warp_sort128_16(a, b);
+        v[0] = a;
+        v[1] = b;
+        v[2] = a >> 16;
+        v[3] = b >> 16;
+    } else {
+        warp_sort128(v);
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) P.slot_order[c * ORDER_CHUNK + lane + 32 * e] = (uint8_t)(v[e] & 127u);
 }
