@@ -286,18 +286,8 @@ __global__ void k_begin(DevParams P, int loop) {
 // fixed (warp-major across blocks, no atomic), later chunks come from a
 // ticket, so warps that drew short rollouts take more work.
 // ---------------------------------------------------------------------------
-#ifndef KPX_QUAD_MIN_BLOCKS
-#define KPX_QUAD_MIN_BLOCKS 3
-#endif
-// resident blocks per SM requested from the register allocator: the 12D
-// quadcopter's RK4 would otherwise need ~100 registers (two blocks per SM)
-template <int DYN>
-struct PropOccupancy {
-    static constexpr int blocks = DYN == KPX_QUAD12 ? KPX_QUAD_MIN_BLOCKS : 4;
-};
-
 template <int DYN, int INTEG, bool SYM>
-__global__ void __launch_bounds__(PROP_THREADS, PropOccupancy<DYN>::blocks)
+__global__ void __launch_bounds__(PropShape<DYN>::threads, PropShape<DYN>::blocks)
     k_propagate(DevParams P, kpx_debug_records rec, int rec_on) {
     pdl_enter();
     kpx_device_header* H = P.hdr;
@@ -590,7 +580,7 @@ int propagate_blocks_per_sm() {
     static int per_sm = 0;
     if (!per_sm) {
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_propagate<DYN, INTEG, SYM>, PROP_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_propagate<DYN, INTEG, SYM>, PropShape<DYN>::threads, 0);
         per_sm = v < 1 ? 1 : v;
     }
     return per_sm;
@@ -607,15 +597,15 @@ template <int DYN, int INTEG>
 cudaError_t launch_propagate_t(const DevParams& P, const kpx_debug_records* rec, cudaStream_t s) {
     const int fit = propagate_occupancy_t<DYN, INTEG>(P, 0);
     const int per_sm = P.prop_bps > 0 && P.prop_bps < fit ? P.prop_bps : fit;
-    const int grid = persistent_blocks((P.slot_cap + PROP_THREADS - 1) / PROP_THREADS, per_sm);
+    const int grid = persistent_blocks((P.slot_cap + PropShape<DYN>::threads - 1) / PropShape<DYN>::threads, per_sm);
     kpx_debug_records r{};
     int on = 0;
     if (rec && rec->valid) {
         r = *rec;
         on = 1;
     }
-    return launch_pdl(P.sym_bounds ? k_propagate<DYN, INTEG, true> : k_propagate<DYN, INTEG, false>, grid, PROP_THREADS,
-                      s, P, r, on);
+    return launch_pdl(P.sym_bounds ? k_propagate<DYN, INTEG, true> : k_propagate<DYN, INTEG, false>, grid,
+                      PropShape<DYN>::threads, s, P, r, on);
 }
 
 template <int DYN, int INTEG>
