@@ -10,6 +10,7 @@
 #include <string>
 #include <algorithm>
 #include <atomic>
+#include <new>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -468,20 +469,60 @@ struct CaptureStreams {
     static constexpr int kDevices = 64;
     cudaStream_t s[kDevices] = {};
     SideBranch side[kDevices];
+    BatchBranches* batch[kDevices] = {};
     ~CaptureStreams() {  // each call fails harmlessly once the context is gone
         for (int d = 0; d < kDevices; ++d) {
             if (s[d]) cudaStreamDestroy(s[d]);
             if (side[d].stream) cudaStreamDestroy(side[d].stream);
             if (side[d].fork) cudaEventDestroy(side[d].fork);
             if (side[d].join) cudaEventDestroy(side[d].join);
+            if (batch[d]) drop(batch[d]);
         }
     }
+    static void drop(BatchBranches* b) {
+        for (cudaStream_t st : b->stream)
+            if (st) cudaStreamDestroy(st);
+        for (cudaEvent_t ev : b->join)
+            if (ev) cudaEventDestroy(ev);
+        if (b->fork) cudaEventDestroy(b->fork);
+        delete b;
+    }
 };
+
+CaptureStreams& capture_streams() {
+    thread_local CaptureStreams streams;
+    return streams;
+}
+
+// The batch branches of this host thread on the current device (made on first
+// use and kept); null when they cannot be made: the classes then run one after
+// another.
+const BatchBranches* batch_branches_here() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= CaptureStreams::kDevices) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    BatchBranches*& kept = capture_streams().batch[dev];
+    if (kept) return kept;
+    BatchBranches* b = new (std::nothrow) BatchBranches{};
+    if (!b) return nullptr;
+    bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (cudaStream_t& st : b->stream) ok = ok && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t& ev : b->join) ok = ok && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        CaptureStreams::drop(b);
+        return nullptr;
+    }
+    kept = b;
+    return b;
+}
 
 // The capture stream and side branch of this host thread on the current
 // device (made on first use and kept); false when they cannot be made.
 bool capture_resources_here(cudaStream_t* stream, SideBranch* side) {
-    thread_local CaptureStreams streams;
+    CaptureStreams& streams = capture_streams();
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= CaptureStreams::kDevices) {
         cudaGetLastError();
@@ -704,12 +745,13 @@ constexpr int kGraphIterations = 8;
 
 cudaError_t capture_batch(kpx_batch* b, int count, cudaGraphExec_t* exec) {
     cudaGraph_t g = nullptr;
+    const BatchBranches* side = batch_branches_here();
     cudaError_t e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return e;
     cudaError_t le = cudaSuccess;
     for (int i = 0; i < count && le == cudaSuccess; ++i)
         le = launch_batch_iteration(b->BP, b->n_classes, b->cls_kind, b->cls_lo, b->cls_hi, b->cls_bps,
-                                    b->capture_stream);
+                                    b->capture_stream, side);
     e = cudaStreamEndCapture(b->capture_stream, &g);
     if (le != cudaSuccess) e = le;
     if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);

@@ -9,6 +9,8 @@
 // prefix sums recomputed every iteration, and a unit finds its problem by a
 // binary search.  Nothing couples two problems, so each result is the one the
 // problem would get alone.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "kpx_phases.cuh"
@@ -96,14 +98,19 @@ __global__ void k_b_snapshot(BatchParams BP) {
         P.region_snap[r] = P.region_key[r];
 }
 
+// As PropShape, with one block fewer for the quadcopter: the problem's
+// parameters come from memory here, not from the constant bank, and at 72
+// registers the kernel spills 328 bytes (2,167 us an iteration of 48 mixed
+// problems; 2,110 at 80 registers, 2,190 at 96).
 template <int DYN>
-struct BatchPropOccupancy {
-    static constexpr int blocks = DYN == KPX_QUAD12 ? 3 : 4;
+struct BatchPropShape {
+    static constexpr int threads = PropShape<DYN>::threads;
+    static constexpr int blocks = DYN == KPX_QUAD12 ? 6 : PropShape<DYN>::blocks;
 };
 
 // propagate over the chunks of the class's problems [lo, hi)
 template <int DYN, int INTEG>
-__global__ void __launch_bounds__(PROP_THREADS, BatchPropOccupancy<DYN>::blocks) k_b_propagate(BatchParams BP) {
+__global__ void __launch_bounds__(BatchPropShape<DYN>::threads, BatchPropShape<DYN>::blocks) k_b_propagate(BatchParams BP) {
     const int64_t c_lo = BP.chunk_prefix[BP.lo], c_hi = BP.chunk_prefix[BP.hi];
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     int64_t chunk = c_lo + (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -120,8 +127,12 @@ __global__ void __launch_bounds__(PROP_THREADS, BatchPropOccupancy<DYN>::blocks)
         const kpx_device_header* H = P.hdr;
         const bool early = (P.flags & KPX_FLAG_EARLY_REJECT) != 0;
         const int64_t unit = propagate_unit_chunk(chunk - BP.chunk_prefix[p], H->n_slots, P.slot_order != nullptr);
-        propagate_chunk<DYN, INTEG>(P, H->n_slots, H->lambda, (uint32_t)H->iter, va_current(P, H), early, unit,
-                                    no_rec, 0, steps, tests, n_valid, P.slot_order);
+        if (P.sym_bounds)
+            propagate_chunk<DYN, INTEG, true>(P, H->n_slots, H->lambda, (uint32_t)H->iter, va_current(P, H), early,
+                                              unit, no_rec, 0, steps, tests, n_valid, P.slot_order);
+        else
+            propagate_chunk<DYN, INTEG, false>(P, H->n_slots, H->lambda, (uint32_t)H->iter, va_current(P, H), early,
+                                               unit, no_rec, 0, steps, tests, n_valid, P.slot_order);
         unsigned long long t = 0ull;
         if ((threadIdx.x & 31) == 0) t = atomicAdd(&BP.bh->prop_ticket[BP.cls], 1ull);
         chunk = c_lo + n_warps + (int64_t)__shfl_sync(FULL, t, 0);
@@ -132,7 +143,16 @@ __global__ void __launch_bounds__(PROP_THREADS, BatchPropOccupancy<DYN>::blocks)
 __global__ void k_b_mark(BatchParams BP) {
     const DevParams& P = BP.Ps[blockIdx.y];
     if (!P.hdr->active) return;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < P.R; r += gridDim.x * blockDim.x) mark_region(P, r);
+    // four regions' keys in flight a thread
+    const int stride = gridDim.x * blockDim.x;
+    for (int r0 = blockIdx.x * blockDim.x + threadIdx.x; r0 < P.R; r0 += 4 * stride) {
+        uint64_t k[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) k[q] = r0 + q * (int64_t)stride < P.R ? P.region_key[r0 + q * stride] : KEY_INF;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k[q] != KEY_INF && (uint32_t)k[q] >= (uint32_t)P.N) mark_region(P, r0 + q * stride);
+    }
 }
 
 __global__ void __launch_bounds__(WIN_THREADS) k_b_scan(BatchParams BP) {
@@ -255,11 +275,11 @@ cudaError_t launch_b_propagate_t(const BatchParams& BP, int bps, cudaStream_t s)
     static int per_sm = 0;
     if (!per_sm) {
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_b_propagate<DYN, INTEG>, PROP_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_b_propagate<DYN, INTEG>, BatchPropShape<DYN>::threads, 0);
         per_sm = v < 1 ? 1 : v;
     }
     const int use = bps > 0 && bps < per_sm ? bps : per_sm;
-    k_b_propagate<DYN, INTEG><<<b_sm_count() * use, PROP_THREADS, 0, s>>>(BP);
+    k_b_propagate<DYN, INTEG><<<b_sm_count() * use, BatchPropShape<DYN>::threads, 0, s>>>(BP);
     return cudaGetLastError();
 }
 
@@ -288,31 +308,51 @@ cudaError_t launch_batch_poll(const BatchParams& base, cudaStream_t s) {
 }
 
 // One batched iteration: begin, snapshot, propagate per class, mark, scan,
-// prefix, append per class, prune, end.
+// prefix, append per class, prune, end.  The classes touch different problems:
+// with side branches (captures) their propagates, and later their appends, run
+// beside one another, so that one class's last rollouts do not leave the GPU
+// to themselves.
 cudaError_t launch_batch_iteration(const BatchParams& base, int n_classes, const int* cls_kind, const int* cls_lo,
-                                   const int* cls_hi, const int* cls_bps, cudaStream_t s) {
+                                   const int* cls_hi, const int* cls_bps, cudaStream_t s, const BatchBranches* side) {
+    // blocks per problem where a grid has a row per problem: enough to fill the
+    // GPU with few problems (a request loop's dozen), at least 8
+    const int row_blocks = std::max(8, (b_sm_count() * 6 + base.B - 1) / base.B);
+    // runs launch(class, its parameters, stream) for every class, the first on s
+    auto per_class = [&](auto launch) -> cudaError_t {
+        cudaError_t e = cudaSuccess;
+        const bool fork = side && n_classes > 1;
+        if (fork) e = cudaEventRecord(side->fork, s);
+        for (int c = 0; c < n_classes && e == cudaSuccess; ++c) {
+            BatchParams bp = base;
+            bp.lo = cls_lo[c];
+            bp.hi = cls_hi[c];
+            bp.cls = c;
+            cudaStream_t sc = s;
+            if (fork && c > 0) {
+                sc = side->stream[c - 1];
+                e = cudaStreamWaitEvent(sc, side->fork, 0);
+            }
+            if (e == cudaSuccess) e = launch(c, bp, sc);
+            if (fork && c > 0 && e == cudaSuccess) e = cudaEventRecord(side->join[c - 1], sc);
+        }
+        for (int c = 1; fork && c < n_classes && e == cudaSuccess; ++c)
+            e = cudaStreamWaitEvent(s, side->join[c - 1], 0);
+        return e;
+    };
     k_b_begin<<<1, 1024, 0, s>>>(base);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_b_snapshot<<<dim3(8, base.B), 256, 0, s>>>(base);
-    for (int c = 0; c < n_classes && e == cudaSuccess; ++c) {
-        BatchParams bp = base;
-        bp.lo = cls_lo[c];
-        bp.hi = cls_hi[c];
-        bp.cls = c;
-        e = [&]() -> cudaError_t { KPX_CLASS_DISPATCH(launch_b_propagate_t, cls_kind[c], bp, cls_bps[c], s); }();
-    }
+    k_b_snapshot<<<dim3(row_blocks, base.B), 256, 0, s>>>(base);
+    e = per_class([&](int c, const BatchParams& bp, cudaStream_t sc) -> cudaError_t {
+        KPX_CLASS_DISPATCH(launch_b_propagate_t, cls_kind[c], bp, cls_bps[c], sc);
+    });
     if (e != cudaSuccess) return e;
-    k_b_mark<<<dim3(8, base.B), 256, 0, s>>>(base);
+    k_b_mark<<<dim3(row_blocks, base.B), 256, 0, s>>>(base);
     k_b_scan<<<b_sm_count() * 8, WIN_THREADS, 0, s>>>(base);
     k_b_prefix<<<1, 1024, 0, s>>>(base);
-    for (int c = 0; c < n_classes && e == cudaSuccess; ++c) {
-        BatchParams bp = base;
-        bp.lo = cls_lo[c];
-        bp.hi = cls_hi[c];
-        bp.cls = c;
-        e = [&]() -> cudaError_t { KPX_CLASS_DISPATCH(launch_b_append_t, cls_kind[c], bp, s); }();
-    }
+    e = per_class([&](int c, const BatchParams& bp, cudaStream_t sc) -> cudaError_t {
+        KPX_CLASS_DISPATCH(launch_b_append_t, cls_kind[c], bp, sc);
+    });
     if (e != cudaSuccess) return e;
     k_b_prune<<<b_sm_count() * 6, PRUNE_THREADS, 0, s>>>(base);  // 40 registers: 6 blocks per SM
     k_b_end<<<(base.B + 255) / 256, 256, 0, s>>>(base);

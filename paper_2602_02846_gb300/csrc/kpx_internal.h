@@ -23,7 +23,6 @@ constexpr uint64_t KEY_INF = ~0ull;
 enum : uint8_t { SET_A = 1, SET_I = 2, SET_T = 3, SET_MASK = 3, SET_ANC = 4, SET_DOM = 8 };
 
 // work partitioning constants
-constexpr int PROP_THREADS = 256;
 constexpr int WIN_THREADS = 256;
 constexpr int WIN_WORDS_PER_THREAD = 8;
 constexpr int WIN_TILE_WORDS = WIN_THREADS * WIN_WORDS_PER_THREAD;   // 2048 words = 65536 slots
@@ -250,9 +249,18 @@ struct BatchParams {
 
 cudaError_t launch_batch_poll(const BatchParams& base, cudaStream_t s);
 
-// cls_bps: per class, propagate blocks per SM (0: as many as fit)
+// Side streams and events with which a captured batch iteration runs its
+// dynamics classes (six at most) on branches of their own.
+struct BatchBranches {
+    cudaStream_t stream[5];
+    cudaEvent_t fork, join[5];
+};
+
+// cls_bps: per class, propagate blocks per SM (0: as many as fit); side: null
+// runs the classes one after another
 cudaError_t launch_batch_iteration(const BatchParams& base, int n_classes, const int* cls_kind, const int* cls_lo,
-                                   const int* cls_hi, const int* cls_bps, cudaStream_t s);
+                                   const int* cls_hi, const int* cls_bps, cudaStream_t s,
+                                   const BatchBranches* side = nullptr);
 
 // launchers (kpx_kernels.cu); each returns the launch status
 cudaError_t launch_init(const DevParams& P, bool first_time, cudaStream_t s);
