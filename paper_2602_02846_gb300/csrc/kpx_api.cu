@@ -248,6 +248,7 @@ void choose_grid(DevParams& P, const float* aabb, int n_obs, float scale = GRID_
         }
         for (int a = 0; a < 3; ++a) {
             P.grid_n[a] = g[a];
+            P.grid_max[a] = (float)(g[a] - 1);
             P.grid_inv[a] = W[a] > 0.0f ? (float)g[a] / W[a] : 0.0f;
         }
         int64_t entries = 0;

@@ -300,10 +300,15 @@ __device__ __forceinline__ void cell_range_ws(const DevParams& P, const GridView
     const float2 txy = __fmul2_rn(__fadd2_rn(make_float2(px, py), make_float2(-P.ws_lo[0], -P.ws_lo[1])),
                                   make_float2(P.grid_inv[0], P.grid_inv[1]));
     const float tz = __fmul_rn(__fsub_rn(pz, P.ws_lo[2]), P.grid_inv[2]);
-    const int cx = (int)fminf(txy.x, (float)(P.grid_n[0] - 1));
-    const int cy = (int)fminf(txy.y, (float)(P.grid_n[1] - 1));
-    const int cz = (int)fminf(tz, (float)(P.grid_n[2] - 1));
-    const int c = (cz * P.grid_n[1] + cy) * P.grid_n[0] + cx;
+    // floor to an integer in the low bits of t + 2^23 rounded down (0 <= t <
+    // 2^23): an add in place of a conversion, which would queue on the
+    // special-function unit; the three biases come off at once
+    constexpr uint32_t BIAS = 0x4B000000u;  // 2^23
+    const uint32_t bx = __float_as_uint(__fadd_rd(fminf(txy.x, P.grid_max[0]), 0x1p23f));
+    const uint32_t by = __float_as_uint(__fadd_rd(fminf(txy.y, P.grid_max[1]), 0x1p23f));
+    const uint32_t bz = __float_as_uint(__fadd_rd(fminf(tz, P.grid_max[2]), 0x1p23f));
+    const uint32_t nx = (uint32_t)P.grid_n[0], ny = (uint32_t)P.grid_n[1];
+    const int c = (int)((bz * ny + by) * nx + bx - BIAS * (ny * nx + nx + 1u));
     if constexpr (SMEM) {
         e0 = G.cell_start[c];
         e1 = min(G.cell_start[c + 1], P.grid_entries);

@@ -82,6 +82,7 @@ struct DevParams {
     // obstacle grid: cell(c, axis a) = clamp(floor((c - ws_lo[a]) * grid_inv[a]), 0, grid_n[a] - 1)
     int32_t grid_n[3];
     float grid_inv[3];
+    float grid_max[3];    // grid_n - 1
     int32_t n_cells;
     int32_t grid_cap;     // entries reserved in cell_box
     int32_t grid_entries; // entries the grid build writes (computed on the host, <= grid_cap)

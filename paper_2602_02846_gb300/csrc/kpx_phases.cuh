@@ -379,10 +379,8 @@ template <bool OBST, bool SMEM, bool SYM, int PL = -1, int ISO = -1, int DYN, in
 __device__ __forceinline__ bool rollout_steps(const DevParams& P, const GridView& G, LaneRollout<DYN, INTEG>& R,
                                               uint32_t& steps, uint32_t& tests) {
     bool ok = true;
-    while (ok && R.k < R.K) {
-        ++steps;
-        ok = R.template advance_in<OBST, SMEM, SYM, PL, ISO>(P, G, tests);
-    }
+    while (ok && R.k < R.K) ok = R.template advance_in<OBST, SMEM, SYM, PL, ISO>(P, G, tests);
+    steps += (uint32_t)R.k;
     return ok;
 }
 
@@ -396,10 +394,7 @@ __device__ __forceinline__ void roll_candidate(const DevParams& P, const GridVie
     C.R.start(P, va, lam, iter, slot);
     bool ok = true;
     if (early) {  // one loop per mode: no per-step test of the flag
-        while (ok && C.R.k < C.R.K) {
-            ++steps;
-            ok = C.R.template advance_in<false, SMEM, SYM>(P, G, tests);
-        }
+        ok = rollout_steps<false, SMEM, SYM>(P, G, C.R, steps, tests);
     } else if (DYN == KPX_QUAD12 && INTEG == KPX_RK4) {  // the cost kind and inertia flag read once
         const bool pl = P.cost_kind == KPX_COST_PATH_LENGTH;
         if (P.iso_inertia) {
