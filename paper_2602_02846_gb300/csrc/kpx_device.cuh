@@ -262,10 +262,22 @@ __device__ __forceinline__ bool bounds_ok(const DevParams& P, const float (&x)[N
 // workspace box.  `tests` accumulates the number of boxes examined.
 // Where the grid is read from: the workspace (global memory, read-only path)
 // or a copy in shared memory (the fused kernel stages small grids).
+// The copy holds a cell's first entry and entry count in one word.
 struct GridView {
     const int32_t* cell_start;
     const float4* cell_box;
 };
+
+constexpr int CELL_START_BITS = 16;
+
+__device__ __forceinline__ int32_t pack_cell(int e0, int e1) {
+    return (int32_t)((uint32_t)e0 | (uint32_t)max(e1 - e0, 0) << CELL_START_BITS);
+}
+
+__device__ __forceinline__ void unpack_cell(int32_t w, int& e0, int& e1) {
+    e0 = w & ((1 << CELL_START_BITS) - 1);
+    e1 = e0 + (int)((uint32_t)w >> CELL_START_BITS);
+}
 
 template <bool SMEM, typename T>
 __device__ __forceinline__ T grid_ld(const T* p) {
@@ -275,20 +287,36 @@ __device__ __forceinline__ T grid_ld(const T* p) {
         return __ldg(p);
 }
 
+// The cell of grid coordinates already clamped to [0, grid_n - 1].  The floor
+// is taken into an integer in the low bits of t + 2^23 rounded down (0 <= t <
+// 2^23): an add in place of a conversion, which would queue on the
+// special-function unit; the three biases come off at once.
+__device__ __forceinline__ int cell_index(const DevParams& P, float tx, float ty, float tz) {
+    constexpr uint32_t BIAS = 0x4B000000u;  // 2^23
+    const uint32_t bx = __float_as_uint(__fadd_rd(tx, 0x1p23f));
+    const uint32_t by = __float_as_uint(__fadd_rd(ty, 0x1p23f));
+    const uint32_t bz = __float_as_uint(__fadd_rd(tz, 0x1p23f));
+    const uint32_t nx = (uint32_t)P.grid_n[0], ny = (uint32_t)P.grid_n[1];
+    return (int)((bz * ny + by) * nx + bx - BIAS * (ny * nx + nx + 1u));
+}
+
 // The entry range [e0, e1) of the point's cell.  Every coordinate, NaN and
 // infinities included, maps to a cell of the grid, so the read stays in
 // range for any point.
 template <bool SMEM>
 __device__ __forceinline__ void cell_range(const DevParams& P, const GridView& G, float px, float py, float pz,
                                            int& e0, int& e1) {
-    const int cx = grid_cell(px, P.ws_lo[0], P.grid_inv[0], P.grid_n[0]);
-    const int cy = grid_cell(py, P.ws_lo[1], P.grid_inv[1], P.grid_n[1]);
-    const int cz = grid_cell(pz, P.ws_lo[2], P.grid_inv[2], P.grid_n[2]);
-    const int c = (cz * P.grid_n[1] + cy) * P.grid_n[0] + cx;
-    // the build keeps every offset within grid_entries <= grid_cap; a
-    // shared-memory copy holds exactly grid_entries boxes
-    e0 = grid_ld<SMEM>(G.cell_start + c);
-    e1 = min(grid_ld<SMEM>(G.cell_start + c + 1), SMEM ? P.grid_entries : P.grid_cap);
+    const float tx = __fmul_rn(__fsub_rn(px, P.ws_lo[0]), P.grid_inv[0]);
+    const float ty = __fmul_rn(__fsub_rn(py, P.ws_lo[1]), P.grid_inv[1]);
+    const float tz = __fmul_rn(__fsub_rn(pz, P.ws_lo[2]), P.grid_inv[2]);
+    const int c = cell_index(P, fminf(fmaxf(tx, 0.0f), P.grid_max[0]), fminf(fmaxf(ty, 0.0f), P.grid_max[1]),
+                             fminf(fmaxf(tz, 0.0f), P.grid_max[2]));
+    if constexpr (SMEM) {
+        unpack_cell(G.cell_start[c], e0, e1);
+    } else {  // the build keeps every offset within grid_entries <= grid_cap
+        e0 = __ldg(G.cell_start + c);
+        e1 = min(__ldg(G.cell_start + c + 1), P.grid_cap);
+    }
 }
 
 // cell_range() for a point inside the workspace box (bounds_ok() passed:
@@ -300,18 +328,9 @@ __device__ __forceinline__ void cell_range_ws(const DevParams& P, const GridView
     const float2 txy = __fmul2_rn(__fadd2_rn(make_float2(px, py), make_float2(-P.ws_lo[0], -P.ws_lo[1])),
                                   make_float2(P.grid_inv[0], P.grid_inv[1]));
     const float tz = __fmul_rn(__fsub_rn(pz, P.ws_lo[2]), P.grid_inv[2]);
-    // floor to an integer in the low bits of t + 2^23 rounded down (0 <= t <
-    // 2^23): an add in place of a conversion, which would queue on the
-    // special-function unit; the three biases come off at once
-    constexpr uint32_t BIAS = 0x4B000000u;  // 2^23
-    const uint32_t bx = __float_as_uint(__fadd_rd(fminf(txy.x, P.grid_max[0]), 0x1p23f));
-    const uint32_t by = __float_as_uint(__fadd_rd(fminf(txy.y, P.grid_max[1]), 0x1p23f));
-    const uint32_t bz = __float_as_uint(__fadd_rd(fminf(tz, P.grid_max[2]), 0x1p23f));
-    const uint32_t nx = (uint32_t)P.grid_n[0], ny = (uint32_t)P.grid_n[1];
-    const int c = (int)((bz * ny + by) * nx + bx - BIAS * (ny * nx + nx + 1u));
+    const int c = cell_index(P, fminf(txy.x, P.grid_max[0]), fminf(txy.y, P.grid_max[1]), fminf(tz, P.grid_max[2]));
     if constexpr (SMEM) {
-        e0 = G.cell_start[c];
-        e1 = min(G.cell_start[c + 1], P.grid_entries);
+        unpack_cell(G.cell_start[c], e0, e1);
     } else {  // the cell's (start, clamped end) pair, one load
         const int2 r = __ldg(P.cell_pair + c);
         e0 = r.x;

@@ -1,7 +1,7 @@
 // kpx_fused.cu -- whole Kino-PAX+ iterations in one launch while the problem
 // is small.
 //
-// With a few thousand slots per iteration, the eight phase kernels are
+// With a few thousand slots per iteration, the seven phase kernels are
 // bound by launch and dependency latency rather than by work: every kernel
 // boundary costs a few microseconds, while the iteration's rollouts need a
 // few in total.  This kernel runs whole iterations inside one thread-block
@@ -21,8 +21,8 @@
 // cluster barriers discard the L1 cache, and every rollout step reads the grid.
 //
 // Before each iteration the leader thread checks that the iteration fits: at
-// most one 32-slot chunk per warp, and a tree of at most FUSED_MAX_NODES
-// nodes.  When it does not fit, the kernel stops and leaves the number of
+// most one slot per thread of the cluster, and a tree of at most
+// FUSED_MAX_NODES nodes.  When it does not fit, the kernel stops and leaves the number of
 // iterations still owed to this graph launch in the header (graph_pending).
 // It then sets the graph's conditional handle, so that the loop of phase
 // kernels that follows it runs them (build_loop_graph in kpx_api.cu).
@@ -34,18 +34,32 @@ namespace kpx {
 
 namespace {
 
-constexpr int FUSED_THREADS = 256;  // = WIN_THREADS = PRUNE_THREADS (block-wide units)
+// Threads of a CTA.  The double integrator and the airplane, whose checks cost
+// several integrations each, split a rollout over lanes of several warps when
+// the slots leave some idle (roll_part): 512 threads on 16 SMs hold 1,024
+// rollouts in eight parts, 4,096 in two, or 8,192 whole.  The rollouts bound
+// these iterations: 200 of the airplane among 300 boxes, 2,944 slots each,
+// take 2.23 ms; 2.33 ms with 256 threads, 2.32 ms unsplit; 2.36 ms with 256
+// threads unsplit, a step integrated ahead of its checks and a cell's two
+// offsets in two words, as it was.  The quadcopter's integration costs more
+// than its checks and needs the registers: 256 threads, and lanes of one warp
+// share the checks (roll_candidate_coop).
+template <int DYN>
+constexpr int FUSED_THREADS = DYN == KPX_QUAD12 ? 256 : 512;
+constexpr int FUSED_MAX_PARTS = 8;
 constexpr int FUSED_MAX_CLUSTER = 16;
 constexpr int FUSED_MAX_NODES = 32768;
 // obstacle grids up to this size are copied into shared memory: every cluster
 // barrier (acquire) discards the L1 cache, and the rollouts read the grid at
 // every step
 constexpr size_t FUSED_GRID_SMEM_MAX = 180 * 1024;
+static_assert(FUSED_GRID_SMEM_MAX / (2 * sizeof(float4)) < (1u << CELL_START_BITS) &&
+                  FUSED_GRID_SMEM_MAX / (2 * sizeof(float4)) < (1u << (32 - CELL_START_BITS)),
+              "pack_cell() holds any entry of a copy");
 
 __host__ __device__ inline size_t grid_start_bytes(int32_t n_cells) {
-    return ((size_t)(n_cells + 1) * sizeof(int32_t) + 15) / 16 * 16;
+    return ((size_t)n_cells * sizeof(int32_t) + 15) / 16 * 16;
 }
-static_assert(FUSED_THREADS == WIN_THREADS && FUSED_THREADS == PRUNE_THREADS, "block-wide units");
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -144,15 +158,18 @@ __device__ __forceinline__ void fused_begin(const DevParams& P, kpx_device_heade
 }
 
 template <int DYN, int INTEG>
-__global__ void __launch_bounds__(FUSED_THREADS, 1)
+__global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     k_fused(DevParams P, int n_iter, cudaGraphConditionalHandle handle, int use_handle, int grid_smem) {
+    constexpr int THREADS = FUSED_THREADS<DYN>, WARPS = THREADS / 32;
+    constexpr bool SPLIT = DYN != KPX_QUAD12;
     extern __shared__ __align__(16) unsigned char fused_grid[];
     __shared__ uint32_t s_prefix;
     __shared__ int32_t s_parent[PRUNE_TILE];
     __shared__ uint8_t s_set[PRUNE_TILE];
     __shared__ uint8_t s_icount[PRUNE_TILE];
     __shared__ uint32_t s_counts[PRUNE_ROUND_WARPS];
-    __shared__ uint32_t s_cnt[FUSED_MAX_CLUSTER * (FUSED_THREADS / 32)];  // winners per chunk (every CTA's copy)
+    __shared__ uint32_t s_cnt[FUSED_MAX_CLUSTER * WARPS];  // winners per chunk (every CTA's copy)
+    __shared__ uint2 s_part[SPLIT ? THREADS : 1];  // a split rollout's parts: steps (top bit: all valid), box tests
     // While the launch runs, the header lives in CTA 0's shared memory: the
     // leader's bookkeeping stays on the SM, and the few header updates of
     // other CTAs (a status, the goal key) reach it over distributed shared
@@ -168,23 +185,25 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
     if (blockIdx.x == 0) {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(P.hdr);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&s_hdr);
-        for (int i = threadIdx.x; i < HDR_WORDS; i += FUSED_THREADS) dst[i] = src[i];
+        for (int i = threadIdx.x; i < HDR_WORDS; i += THREADS) dst[i] = src[i];
         __syncthreads();
     }
     kpx_device_header* H = dsmem_generic(&s_hdr, 0);
     const int lane = threadIdx.x & 31;
     const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
     const int n_cta = (int)gridDim.x;  // the grid is one cluster
-    const int64_t gtid = (int64_t)blockIdx.x * FUSED_THREADS + threadIdx.x;
-    const int64_t gthreads = (int64_t)n_cta * FUSED_THREADS;
-    const int n_chunks = n_cta * (FUSED_THREADS / 32);  // one per warp of the cluster
+    const int64_t gtid = (int64_t)blockIdx.x * THREADS + threadIdx.x;
+    const int64_t gthreads = (int64_t)n_cta * THREADS;
     const bool early = (P.flags & KPX_FLAG_EARLY_REJECT) != 0;
     GridView G{P.cell_start, P.cell_box};
     if (grid_smem) {  // the obstacle grid is read-only while planning
         int32_t* sc = reinterpret_cast<int32_t*>(fused_grid);
         float4* sb = reinterpret_cast<float4*>(fused_grid + grid_start_bytes(P.n_cells));
-        for (int i = threadIdx.x; i <= P.n_cells; i += FUSED_THREADS) sc[i] = P.cell_start[i];
-        for (int i = threadIdx.x; i < 2 * P.grid_entries; i += FUSED_THREADS) sb[i] = P.cell_box[i];
+        for (int i = threadIdx.x; i < P.n_cells; i += THREADS) {
+            const int2 r = P.cell_pair[i];
+            sc[i] = pack_cell(min(r.x, P.grid_entries), min(r.y, P.grid_entries));
+        }
+        for (int i = threadIdx.x; i < 2 * P.grid_entries; i += THREADS) sb[i] = P.cell_box[i];
         __syncthreads();
         G = GridView{sc, sb};
     }
@@ -223,19 +242,49 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
             for (int64_t r = gtid; r < P.R; r += gthreads) P.region_snap[r] = P.region_key[r];
             cluster_barrier();
         }
-        // propagate (Alg. 2): one chunk of 32 / g slots per warp, warp-major
-        // across the CTAs; g lanes share a rollout when the slots fill at
-        // most half of the cluster's threads.  The lane that keeps a
-        // candidate holds it in registers.
-        const int g = early ? 1 : coop_lanes(n_slots, gthreads);
-        const int64_t chunk = (int64_t)(threadIdx.x >> 5) * n_cta + blockIdx.x;
+        // propagate (Alg. 2): chunks of slots, warp-major across the CTAs.
+        // When the slots leave threads idle, a rollout is split over lanes of
+        // `parts` warps (roll_part), a chunk being 32 slots; or (the
+        // quadcopter) g lanes of a warp share it, a chunk being 32 / g slots.
+        // The lane that keeps a candidate holds it in registers.
+        const int g = SPLIT || early ? 1 : coop_lanes(n_slots, gthreads);
+        int parts = 1;
+        if (SPLIT && !early)
+            while (parts < FUSED_MAX_PARTS && n_slots * (2 * parts) <= gthreads) parts *= 2;
+        const int warp = threadIdx.x >> 5;
+        const int n_chunks = n_cta * (WARPS / parts);
+        const int64_t chunk = (int64_t)(warp / parts) * n_cta + blockIdx.x;
+        const int part = warp % parts;
         const int64_t slot = chunk * (32 / g) + lane / g;
         Candidate<DYN, INTEG> C;
         C.ok = false;
         {
             uint32_t steps = 0, tests = 0, n_valid = 0;
             const bool live = slot < n_slots;
-            if (g > 1) {  // all lanes of the warp take part
+            if (SPLIT && parts > 1) {
+                bool ok = false;
+                if (live) {
+                    C.R.start(P, va, lam, iter, slot);
+                    const int k0 = split_point<DYN>(C.R.K, part, parts), k1 = split_point<DYN>(C.R.K, part + 1, parts);
+                    if (grid_smem)
+                        ok = roll_part<DYN, INTEG, true>(P, G, C.R, k0, k1, steps, tests);
+                    else
+                        ok = roll_part<DYN, INTEG, false>(P, G, C.R, k0, k1, steps, tests);
+                    s_part[threadIdx.x] = make_uint2(steps | (ok ? 0x80000000u : 0u), tests);
+                    steps = tests = 0;
+                }
+                __syncthreads();
+                if (live && part == parts - 1) {  // the last part has the end state
+                    ok = true;
+                    for (int q = 0; q < parts && ok; ++q) {  // up to the first part that failed
+                        const uint2 r = s_part[((warp / parts) * parts + q) * 32 + lane];
+                        steps += r.x & 0x7FFFFFFFu;
+                        tests += r.y;
+                        ok = (r.x >> 31) != 0u;
+                    }
+                    finish_candidate<DYN, INTEG>(P, slot, ok, C);
+                }
+            } else if (g > 1) {  // all lanes of the warp take part
                 if (grid_smem)
                     roll_candidate_coop<DYN, INTEG, true>(P, G, lam, iter, va, live, slot, g, C, steps, tests);
                 else
@@ -246,7 +295,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
                         roll_candidate<DYN, INTEG, true>(P, G, lam, iter, va, true, slot, C, steps, tests);
                     else
                         roll_candidate<DYN, INTEG, false>(P, G, lam, iter, va, true, slot, C, steps, tests);
-                } else if (DYN == KPX_DI6) {  // a short step: nothing to overlap
+                } else if (SPLIT) {  // 16 warps: nothing to overlap
                     if (grid_smem)
                         roll_candidate<DYN, INTEG, true>(P, G, lam, iter, va, false, slot, C, steps, tests);
                     else
@@ -282,9 +331,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
         // CTA 0 prunes tile 0: it stages the tile now, in the same round
         // trip, and the winners that take a region from one of its nodes
         // write that node's new set byte into the staged copy as well
-        if (blockIdx.x == 0) stage_tile(P, 0, n_old, s_parent, s_set, s_icount);
+        if (blockIdx.x == 0) stage_tile<THREADS>(P, 0, n_old, s_parent, s_set, s_icount);
         const uint32_t word = __ballot_sync(FULL, won);
-        if (lane < n_cta) dsmem_store(s_cnt + chunk, (uint32_t)lane, (uint32_t)__popc(word));
+        if (lane < n_cta && part == parts - 1) dsmem_store(s_cnt + chunk, (uint32_t)lane, (uint32_t)__popc(word));
         cluster_barrier();
         // the winners kept: every thread derives them alike (prune uses them
         // too, so it reads no header field the leader may rewrite at its end)
@@ -324,7 +373,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
         // so only the launch's last iteration reaches it, at the end
         pA = pI = pT = 0;
         for (int t = blockIdx.x; t < n_tiles; t += n_cta)
-            prune_tile(P, H, (uint32_t)t, n_tiles, n_old, total, epoch, va_next, s_parent, s_set, s_icount, s_counts,
+            prune_tile<THREADS>(P, H, (uint32_t)t, n_tiles, n_old, total, epoch, va_next, s_parent, s_set, s_icount, s_counts,
                        s_prefix, pA, pI, pT, t == 0);
         ++done;
         if (merged && lead_warp) {  // prune_tile ended with a CTA barrier
@@ -355,7 +404,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
     if (blockIdx.x == 0) {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&s_hdr);
         uint32_t* dst = reinterpret_cast<uint32_t*>(P.hdr);
-        for (int i = threadIdx.x; i < HDR_WORDS; i += FUSED_THREADS) dst[i] = src[i];
+        for (int i = threadIdx.x; i < HDR_WORDS; i += THREADS) dst[i] = src[i];
         if (leader && use_handle) cudaGraphSetConditional(handle, s_hdr.graph_pending > 0 ? 1u : 0u);
     }
 }
@@ -376,7 +425,7 @@ int fused_cluster_size_t(const DevParams&, int) {
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(FUSED_MAX_CLUSTER);
-        cfg.blockDim = dim3(FUSED_THREADS);
+        cfg.blockDim = dim3(FUSED_THREADS<DYN>);
         cfg.dynamicSmemBytes = FUSED_GRID_SMEM_MAX;  // the cluster must fit with a staged grid
         int cl = 0;
         if (cudaOccupancyMaxPotentialClusterSize(&cl, (const void*)k_fused<DYN, INTEG>, &cfg) != cudaSuccess) {
@@ -400,7 +449,7 @@ cudaError_t launch_fused_t(const DevParams& P, int n_iter, cudaGraphConditionalH
     const int grid_smem = P.n_obs > 0 && grid_bytes <= FUSED_GRID_SMEM_MAX ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(FUSED_THREADS);
+    cfg.blockDim = dim3(FUSED_THREADS<DYN>);
     cfg.dynamicSmemBytes = grid_smem ? grid_bytes : 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];

@@ -434,8 +434,26 @@ __device__ __forceinline__ void roll_candidate(const DevParams& P, const GridVie
     C.ok = ok;
 }
 
+// A rolled-out candidate's region, cost and key, with the region's atomicMin
+// done, when all its points were valid.
+template <int DYN, int INTEG>
+__device__ __forceinline__ void finish_candidate(const DevParams& P, int64_t slot, bool ok, Candidate<DYN, INTEG>& C) {
+    C.r = -1;
+    C.c = 0.0f;
+    C.key = KEY_INF;
+    if (ok) {
+        C.r = region_of<Dims<DYN>::n>(P, C.R.x);
+        C.c = C.R.cost(P);
+        C.key = pack_key(C.c, (uint32_t)P.N + (uint32_t)slot);
+        if (C.key < __ldcg(&P.region_key[C.r]))
+            atomicMin((unsigned long long*)&P.region_key[C.r], (unsigned long long)C.key);
+    }
+    C.ok = ok;
+}
+
 // roll_candidate() with early reject off, for one lane whose warp waits on
-// its longest rollout (the fused kernel): step k+1 is integrated before step
+// its longest rollout (the quadcopter in the fused kernel, a few warps an SM):
+// step k+1 is integrated before step
 // k's point is checked, so that the integration and the check, which both
 // depend only on step k's state, overlap instead of the check's verdict
 // gating the next integration.  The bounds test does not short-circuit the
@@ -474,17 +492,46 @@ __device__ __forceinline__ void roll_candidate_ahead(const DevParams& P, const G
             break;
         }
     }
-    C.r = -1;
-    C.c = 0.0f;
-    C.key = KEY_INF;
-    if (ok) {
-        C.r = region_of<n>(P, C.R.x);
-        C.c = C.R.cost(P);
-        C.key = pack_key(C.c, (uint32_t)P.N + (uint32_t)slot);
-        if (C.key < __ldcg(&P.region_key[C.r]))
-            atomicMin((unsigned long long*)&P.region_key[C.r], (unsigned long long)C.key);
+    finish_candidate<DYN, INTEG>(P, slot, ok, C);
+}
+
+// A rollout split over P lanes in P warps (the fused kernel, when its slots
+// leave threads idle): part p integrates up to its first step without checks,
+// then checks its own steps, so the longest rollout's checks, which cost
+// several integrations each, run in P places at once.  UNCHECKED_COST: the
+// cost of an unchecked step over a checked one; the parts' steps fall by the
+// factor 1 - UNCHECKED_COST, so that all end together (any split gives the
+// same results).
+template <int DYN>
+constexpr float UNCHECKED_COST = DYN == KPX_DI6 ? 0.04f : 0.24f;
+
+// the steps of a K-step rollout before part p of P
+template <int DYN>
+__device__ __forceinline__ int split_point(int K, int p, int P) {
+    float w = 1.0f, before = 0.0f, all = 0.0f;
+    for (int q = 0; q < P; ++q) {
+        if (q < p) before += w;
+        all += w;
+        w *= 1.0f - UNCHECKED_COST<DYN>;
     }
-    C.ok = ok;
+    return p == P ? K : (int)((float)K * (before / all) + 0.5f);
+}
+
+// One part: steps k0 + 1 .. k1 checked; returns whether all were valid, with
+// the steps and box tests done.  R ends at step k1's state when they were.
+// The checks follow their step one after another: the warps of the other
+// parts fill the waits, and a step integrated ahead (roll_candidate_ahead())
+// only adds instructions (the Dubins forest's iterations: 2.28 ms against
+// 2.33 ms ahead).
+template <int DYN, int INTEG, bool SMEM>
+__device__ __forceinline__ bool roll_part(const DevParams& P, const GridView& G, LaneRollout<DYN, INTEG>& R, int k0,
+                                          int k1, uint32_t& steps, uint32_t& tests) {
+    for (int k = 0; k < k0; ++k) R.integrate(P);
+    for (int k = k0; k < k1; ++k) {
+        ++steps;
+        if (!R.template advance_in<true, SMEM>(P, G, tests)) return false;
+    }
+    return true;
 }
 
 // Lanes per rollout for n_slots rollouts on `threads` threads: the largest
@@ -908,9 +955,11 @@ __device__ __forceinline__ bool prune_rules_123(uint8_t sb, int i_max, int& ic, 
 // The tile's parent ids, set bytes and inactivity counts below n_old, read in
 // one pass: ancestor walks that stay inside the tile read shared memory
 // (parents precede children), and a node's own bytes come from here.
+// THREADS: the block's (k_fused has more than PRUNE_THREADS for some systems)
+template <int THREADS>
 __device__ __forceinline__ void stage_tile(const DevParams& P, int tile0, int n_old, int32_t* s_parent,
                                            uint8_t* s_set, uint8_t* s_icount) {
-    for (int k = threadIdx.x; k < PRUNE_TILE; k += PRUNE_THREADS) {
+    for (int k = threadIdx.x; k < PRUNE_TILE; k += THREADS) {
         const int i = tile0 + k;
         const bool in = i < n_old;
         s_parent[k] = in ? P.parent[i] : -1;
@@ -921,30 +970,32 @@ __device__ __forceinline__ void stage_tile(const DevParams& P, int tile0, int n_
 
 // staged: the caller staged the tile already (the fused kernel stages tile 0
 // before the append phase, whose dominated marks it then receives directly).
-// One pass, one node per thread in each of PRUNE_PER_THREAD rounds (node
-// tile0 + round * PRUNE_THREADS + thread): rules 1-3, then rule 4's walk
+// One pass, one node per thread in each of PRUNE_TILE / THREADS rounds (node
+// tile0 + round * THREADS + thread): rules 1-3, then rule 4's walk
 // for the nodes they leave undecided, so that a small tree's nodes spread
 // over the block's warps.  The compaction keeps id order, which runs round
 // by round, then warp by warp, then lane by lane: each warp ballots its
 // active nodes of each round, and one warp scans the (round, warp) counts,
 // PRUNE_ROUND_WARPS of them, in that order (s_counts) and takes the tile's
 // look-back.
-constexpr int PRUNE_ROUND_WARPS = PRUNE_PER_THREAD * (PRUNE_THREADS / 32);
+constexpr int PRUNE_ROUND_WARPS = PRUNE_TILE / 32;
 static_assert(PRUNE_ROUND_WARPS <= 32, "one warp scans the (round, warp) counts");
 
+template <int THREADS = PRUNE_THREADS>
 __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header* H, uint32_t tile, int n_tiles,
                                            int n_old, int total, uint32_t epoch, int32_t* va_next,
                                            int32_t* s_parent, uint8_t* s_set, uint8_t* s_icount,
                                            uint32_t* s_counts, uint32_t& s_prefix, int& cA, int& cI, int& cT,
                                            bool staged = false) {
+    constexpr int PER = PRUNE_TILE / THREADS;
     const int i_max = P.i_max;
     const int tile0 = (int)tile * PRUNE_TILE;
-    if (!staged) stage_tile(P, tile0, n_old, s_parent, s_set, s_icount);
+    if (!staged) stage_tile<THREADS>(P, tile0, n_old, s_parent, s_set, s_icount);
     __syncthreads();
     uint32_t fields = 0;  // bit q: this thread's node of round q stays in V_A
 #pragma unroll
-    for (int q = 0; q < PRUNE_PER_THREAD; ++q) {
-        const int k = threadIdx.x + q * PRUNE_THREADS;
+    for (int q = 0; q < PER; ++q) {
+        const int k = threadIdx.x + q * THREADS;
         const int i = tile0 + k;
         if (i >= total) continue;
         if (i >= n_old) {  // appended this iteration: in V_A
@@ -1006,11 +1057,11 @@ __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header
         }
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t ball[PRUNE_PER_THREAD];
+    uint32_t ball[PER];
 #pragma unroll
-    for (int q = 0; q < PRUNE_PER_THREAD; ++q) {
+    for (int q = 0; q < PER; ++q) {
         ball[q] = __ballot_sync(FULL, (fields >> q) & 1u);
-        if (lane == 0) s_counts[q * (PRUNE_THREADS / 32) + warp] = (uint32_t)__popc(ball[q]);
+        if (lane == 0) s_counts[q * (THREADS / 32) + warp] = (uint32_t)__popc(ball[q]);
     }
     __syncthreads();
     if (warp == 0) {
@@ -1035,13 +1086,13 @@ __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header
     __syncthreads();
     const uint32_t lt = (1u << lane) - 1u;  // lanes below this one
 #pragma unroll
-    for (int q = 0; q < PRUNE_PER_THREAD; ++q) {
+    for (int q = 0; q < PER; ++q) {
         if ((fields >> q) & 1u) {
             // at most one active node per region, so pos < min(N, R) = va_cap
             const uint32_t pos =
-                s_prefix + s_counts[q * (PRUNE_THREADS / 32) + warp] + (uint32_t)__popc(ball[q] & lt);
+                s_prefix + s_counts[q * (THREADS / 32) + warp] + (uint32_t)__popc(ball[q] & lt);
             if (pos < (uint32_t)P.va_cap)
-                va_next[pos] = tile0 + (int)threadIdx.x + q * PRUNE_THREADS;
+                va_next[pos] = tile0 + (int)threadIdx.x + q * THREADS;
             else
                 set_status(H, KPX_E_INTERNAL);
         }
