@@ -667,10 +667,10 @@ __device__ __forceinline__ int64_t propagate_unit_chunk(int64_t q, int64_t n_slo
 // Threads of a propagate block and the resident blocks per SM asked of the
 // register allocator.  The quadcopter's RK4 is bound by issue with stalls on
 // the FMA, special-function and load pipes between; it would take ~100
-// registers.  Seven blocks of 128 threads at 72 registers (28 warps an SM, 28
-// bytes spilled) beat three of 256 at 80 (24 warps): 0.249 against 0.256 ms a
-// launch in the building; eight at 64 registers spill 168 bytes and take
-// 0.251, six 0.255, two of 256 0.277.
+// registers.  Seven blocks of 128 threads at 72 registers (28 warps an SM) beat
+// three of 256 at 80 (24 warps): 0.249 against 0.256 ms a launch in the
+// building; eight at 64 registers, with spills, take 0.251, six 0.255, two of
+// 256 0.277 (0.234 since, with the stage sums of quad_fma()).
 template <int DYN>
 struct PropShape {
     static constexpr int threads = DYN == KPX_QUAD12 ? 128 : 256;
