@@ -36,9 +36,10 @@ namespace {
 
 // Threads of a CTA.  The double integrator and the airplane, whose checks cost
 // several integrations each, split a rollout over lanes of several warps when
-// the slots leave some idle (roll_part): 512 threads on 16 SMs hold 1,024
-// rollouts in eight parts, 4,096 in two, or 8,192 whole.  The rollouts bound
-// these iterations: 200 of the airplane among 300 boxes, 2,944 slots each,
+// the slots leave some idle (roll_part): 512 threads on 16 SMs hold 2,048
+// rollouts in four parts, 4,096 in two, or 8,192 whole.  Eight parts cost more
+// unchecked steps than they save checks (200 iterations of 576 slots: 2.04 ms
+// against 1.83 ms in four).  The rollouts bound these iterations: 200 of the airplane among 300 boxes, 2,944 slots each,
 // take 2.23 ms; 2.33 ms with 256 threads, 2.32 ms unsplit; 2.36 ms with 256
 // threads unsplit, a step integrated ahead of its checks and a cell's two
 // offsets in two words, as it was.  The quadcopter's integration costs more
@@ -46,7 +47,7 @@ namespace {
 // share the checks (roll_candidate_coop).
 template <int DYN>
 constexpr int FUSED_THREADS = DYN == KPX_QUAD12 ? 256 : 512;
-constexpr int FUSED_MAX_PARTS = 8;
+constexpr int FUSED_MAX_PARTS = 4;
 constexpr int FUSED_MAX_CLUSTER = 16;
 constexpr int FUSED_MAX_NODES = 32768;
 // obstacle grids up to this size are copied into shared memory: every cluster
