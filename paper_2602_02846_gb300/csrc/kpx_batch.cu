@@ -151,7 +151,7 @@ __global__ void k_b_mark(BatchParams BP) {
         for (int q = 0; q < 4; ++q) k[q] = r0 + q * (int64_t)stride < P.R ? P.region_key[r0 + q * stride] : KEY_INF;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (k[q] != KEY_INF && (uint32_t)k[q] >= (uint32_t)P.N) mark_region(P, r0 + q * stride);
+            if (k[q] != KEY_INF && (uint32_t)k[q] >= (uint32_t)P.N) mark_region(P, r0 + q * stride, k[q]);
     }
 }
 
@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(WIN_THREADS) k_b_scan(BatchParams BP) {
         const DevParams& P = BP.Ps[p];
         kpx_device_header* H = P.hdr;
         const int64_t n_tiles = BP.scan_prefix[p + 1] - BP.scan_prefix[p];
-        scan_tile(P, H, (uint32_t)(t - BP.scan_prefix[p]), n_tiles, (H->n_slots + 31) / 32, WIN_WORDS_PER_THREAD, s_warp,
-                  s_prefix);
+        scan_tile(P, H, (uint32_t)(t - BP.scan_prefix[p]), n_tiles, (H->n_slots + 31) / 32, WIN_WORDS_PER_THREAD,
+                  (uint32_t)H->epoch, s_warp, s_prefix);
     }
 }
 

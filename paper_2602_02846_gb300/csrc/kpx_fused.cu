@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
         // so only the launch's last iteration reaches it, at the end
         pA = pI = pT = 0;
         for (int t = blockIdx.x; t < n_tiles; t += n_cta)
-            prune_tile<THREADS>(P, H, (uint32_t)t, n_tiles, n_old, total, epoch, va_next, s_parent, s_set, s_icount, s_counts,
-                       s_prefix, pA, pI, pT, t == 0);
+            prune_tile<THREADS, false>(P, H, (uint32_t)t, n_tiles, n_old, total, epoch, va_next, s_parent, s_set,
+                                       s_icount, s_counts, s_prefix, pA, pI, pT, t == 0);
         ++done;
         if (merged && lead_warp) {  // prune_tile ended with a CTA barrier
             if (leader) {

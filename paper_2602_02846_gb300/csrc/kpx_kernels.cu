@@ -49,6 +49,32 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The header's words that a phase starts from, read together: one round trip
+// to L2 before its first dependent load, where a test of `active` ahead of the
+// other reads made it two (the loads are volatile so that they stay there).
+// Words that this or a concurrent kernel writes are read but not used.
+template <int Q>
+__device__ __forceinline__ int4 header_quad(const kpx_device_header* H) {
+    int4 v;
+    asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(reinterpret_cast<const int4*>(H) + Q));
+    return v;
+}
+static_assert(offsetof(kpx_device_header, status) == 0 && offsetof(kpx_device_header, active) == 4 &&
+                  offsetof(kpx_device_header, iter) == 8 && offsetof(kpx_device_header, n_nodes) == 12,
+              "quad 0");
+static_assert(offsetof(kpx_device_header, lambda) == 20 && offsetof(kpx_device_header, va_sel) == 24, "quad 1");
+static_assert(offsetof(kpx_device_header, n_slots) == 32, "quad 2");
+static_assert(offsetof(kpx_device_header, n_win) == 48 && offsetof(kpx_device_header, n_kept) == 52 &&
+                  offsetof(kpx_device_header, epoch) == 60,
+              "quad 3");
+static_assert(offsetof(kpx_device_header, win_ticket) == 72, "quad 4");
+
+__device__ __forceinline__ int64_t quad_int64(const int4& v) {
+    return (int64_t)((uint64_t)(uint32_t)v.x | (uint64_t)(uint32_t)v.y << 32);
+}
+
 // ---------------------------------------------------------------------------
 // init / reset: Alg. 1 initialisation.
 // ---------------------------------------------------------------------------
@@ -256,6 +282,8 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
 __global__ void k_begin(DevParams P, int loop) {
     pdl_enter();
     kpx_device_header* H = P.hdr;
+    (void)header_quad<0>(H);  // with the next one: the reads below then hit L1
+    (void)header_quad<1>(H);
     const bool allowed = !loop || H->graph_pending > 0;
     const bool snap = begin_needs_snapshot(P, H, allowed);  // reads counters begin_counters leaves alone
     const bool runs = allowed && problem_runs(P, H);
@@ -291,11 +319,12 @@ __global__ void __launch_bounds__(PropShape<DYN>::threads, PropShape<DYN>::block
     k_propagate(DevParams P, kpx_debug_records rec, int rec_on) {
     pdl_enter();
     kpx_device_header* H = P.hdr;
-    if (!H->active) return;
-    const int64_t n_slots = H->n_slots;
-    const int lam = H->lambda;
-    const uint32_t iter = (uint32_t)H->iter;
-    const int32_t* va = va_current(P, H);
+    const int4 h0 = header_quad<0>(H), h1 = header_quad<1>(H), h2 = header_quad<2>(H);
+    if (!h0.y) return;  // not active
+    const int64_t n_slots = quad_int64(h2);
+    const int lam = h1.y;
+    const uint32_t iter = (uint32_t)h0.z;
+    const int32_t* va = h1.z ? P.va1 : P.va0;  // va_current()
     const bool early = (P.flags & KPX_FLAG_EARLY_REJECT) && !rec_on;
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const bool ordered = P.slot_order != nullptr;
@@ -315,8 +344,12 @@ __global__ void __launch_bounds__(PropShape<DYN>::threads, PropShape<DYN>::block
 
 __global__ void k_mark(DevParams P) {
     pdl_enter();
-    if (!P.hdr->active) return;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < P.R; r += gridDim.x * blockDim.x) mark_region(P, r);
+    const int active = P.hdr->active;
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < P.R; r += gridDim.x * blockDim.x) {
+        const uint64_t k = P.region_key[r];  // with the header's word, not after it
+        if (!active) return;
+        mark_region(P, r, k);
+    }
 }
 
 __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
@@ -324,8 +357,10 @@ __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
     __shared__ uint32_t s_tile, s_prefix;
     __shared__ uint32_t s_warp[WIN_THREADS / 32];
     kpx_device_header* H = P.hdr;
-    if (!H->active) return;
-    const int64_t live_words = (H->n_slots + 31) / 32;
+    const int4 h0 = header_quad<0>(H), h2 = header_quad<2>(H), h3 = header_quad<3>(H);
+    if (!h0.y) return;
+    const uint32_t epoch = (uint32_t)h3.w;
+    const int64_t live_words = (quad_int64(h2) + 31) / 32;
     const int per = scan_words_per_thread(P, live_words);
     const int64_t n_tiles = scan_tiles(live_words, per);
     if ((int64_t)blockIdx.x >= n_tiles) return;  // the other blocks take every tile
@@ -335,7 +370,8 @@ __global__ void __launch_bounds__(WIN_THREADS) k_scan(DevParams P) {
         const uint32_t tile = s_tile;
         __syncthreads();
         if ((int64_t)tile >= n_tiles) return;
-        scan_tile(P, H, tile, n_tiles, live_words, per, s_warp, s_prefix);
+        scan_tile(P, H, tile, n_tiles, live_words, per, epoch, s_warp, s_prefix);
+        if (n_tiles <= (int64_t)gridDim.x) return;  // a tile a block: no second ticket
     }
 }
 
@@ -343,9 +379,10 @@ template <int DYN, int INTEG>
 __global__ void __launch_bounds__(128) k_append(DevParams P) {
     pdl_enter();
     kpx_device_header* H = P.hdr;
-    if (!H->active) return;
-    const int W = H->n_win;
-    const int n_old = H->n_nodes;
+    const int4 h0 = header_quad<0>(H), h1 = header_quad<1>(H), h3 = header_quad<3>(H);
+    if (!h0.y) return;
+    const int W = h3.x;
+    const int n_old = h0.w;
     const int room = P.N - n_old;
     const int kept = W < room ? W : room;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -356,9 +393,9 @@ __global__ void __launch_bounds__(128) k_append(DevParams P) {
         // that starts late may find the iteration already ended)
         H->win_ticket = (uint32_t)((n_old + kept + PRUNE_TILE - 1) / PRUNE_TILE);
     }
-    const int lam = H->lambda;
-    const uint32_t iter = (uint32_t)H->iter;
-    const int32_t* va = va_current(P, H);
+    const int lam = h1.y;
+    const uint32_t iter = (uint32_t)h0.z;
+    const int32_t* va = h1.z ? P.va1 : P.va0;
     for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < W; w += gridDim.x * blockDim.x)
         append_meta<DYN, INTEG>(P, H, w, kept, n_old, lam, iter, va);
 }
@@ -403,21 +440,22 @@ template <int DYN, int INTEG>
 __global__ void __launch_bounds__(STAGE_THREADS) k_stage(DevParams P, LoopEnd E) {
     pdl_enter();
     kpx_device_header* H = P.hdr;
-    if (!H->active) {
+    const int4 h0 = header_quad<0>(H), h1 = header_quad<1>(H), h3 = header_quad<3>(H);
+    if (!h0.y) {
         if (blockIdx.x == 0) finish_block(P, E, 2);
         return;
     }
-    const int W = H->n_win;
-    const int n_old = H->n_nodes;  // end_counters advances it only after both halves
+    const int W = h3.x;
+    const int n_old = h0.w;  // end_counters advances it only after both halves
     const int room = P.N - n_old;
     const int kept = W < room ? W : room;
     // A block that starts after the iteration's end (it has no work, so the end
     // did not wait for it) sees less room and so still no work.
     const int working = working_blocks((int)gridDim.x, (kept + STAGE_THREADS - 1) / STAGE_THREADS);
     if ((int)blockIdx.x >= working) return;
-    const int lam = H->lambda;
-    const uint32_t iter = (uint32_t)H->iter;
-    const int32_t* va = va_current(P, H);
+    const int lam = h1.y;
+    const uint32_t iter = (uint32_t)h0.z;
+    const int32_t* va = h1.z ? P.va1 : P.va0;
     const int tiles = (n_old + kept + PRUNE_TILE - 1) / PRUNE_TILE;
     for (int w = blockIdx.x * STAGE_THREADS + threadIdx.x; w < kept; w += gridDim.x * STAGE_THREADS)
         stage_winner<DYN, INTEG>(P, H, w, n_old, lam, iter, va);
@@ -432,17 +470,18 @@ __global__ void __launch_bounds__(PRUNE_THREADS, 8) k_prune(DevParams P, LoopEnd
     __shared__ uint8_t s_icount[PRUNE_TILE];
     __shared__ uint32_t s_counts[PRUNE_ROUND_WARPS];
     kpx_device_header* H = P.hdr;
-    if (!H->active) {
+    const int4 h0 = header_quad<0>(H), h1 = header_quad<1>(H), h3 = header_quad<3>(H), h4 = header_quad<4>(H);
+    if (!h0.y) {
         if (blockIdx.x == 0) finish_block(P, E, 2);
         return;
     }
-    const int n_tiles = (int)H->win_ticket;  // append's
+    const int n_tiles = h4.z;  // append's
     if ((int)blockIdx.x >= n_tiles) return;  // the other blocks take every tile
-    const int n_old = H->n_nodes;
-    const int kept = H->n_kept;
+    const int n_old = h0.w;
+    const int kept = h3.y;
     const int total = n_old + kept;
-    const uint32_t epoch = (uint32_t)H->epoch;
-    int32_t* va_next = va_following(P, H);
+    const uint32_t epoch = (uint32_t)h3.w;
+    int32_t* va_next = h1.z ? P.va0 : P.va1;  // va_following()
     int cA = 0, cI = 0, cT = 0;
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(&H->prune_ticket, 1u);
@@ -452,6 +491,7 @@ __global__ void __launch_bounds__(PRUNE_THREADS, 8) k_prune(DevParams P, LoopEnd
         if ((int)tile >= n_tiles) break;
         prune_tile(P, H, tile, n_tiles, n_old, total, epoch, va_next, s_parent, s_set, s_icount, s_counts, s_prefix,
                    cA, cI, cT);
+        if (n_tiles <= (int)gridDim.x) break;  // a tile a block: no second ticket
     }
     flush_prune_counters(H, cA, cI, cT);
     finish_block(P, E, working_blocks((int)gridDim.x, n_tiles) +

@@ -699,8 +699,8 @@ __device__ __forceinline__ void flush_propagate_counters(kpx_device_header* H, u
 // mark: a region whose key carries a candidate id (>= N) names the slot of
 // the winner of that region (the V_U filter: "cost(x) = cost(R_i)").
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void mark_region(const DevParams& P, int r) {
-    const uint64_t k = P.region_key[r];
+// k: region r's key
+__device__ __forceinline__ void mark_region(const DevParams& P, int r, uint64_t k) {
     if (k == KEY_INF) return;
     const uint32_t id = (uint32_t)k;
     if (id < (uint32_t)P.N) return;
@@ -735,7 +735,8 @@ __device__ __forceinline__ int64_t scan_tiles(int64_t live_words, int per) {
 }
 
 __device__ __forceinline__ void scan_tile(const DevParams& P, kpx_device_header* H, uint32_t tile, int64_t n_tiles,
-                                          int64_t live_words, int per, uint32_t* s_warp, uint32_t& s_prefix) {
+                                          int64_t live_words, int per, uint32_t epoch, uint32_t* s_warp,
+                                          uint32_t& s_prefix) {
     const int64_t w0 = ((int64_t)tile * WIN_THREADS + threadIdx.x) * per;
     static_assert(WIN_WORDS_PER_THREAD == 8, "two 16-byte loads a thread");
     uint32_t w[WIN_WORDS_PER_THREAD];
@@ -755,7 +756,7 @@ __device__ __forceinline__ void scan_tile(const DevParams& P, kpx_device_header*
     uint32_t agg;
     const uint32_t excl = block_exclusive_scan<WIN_THREADS>(cnt, agg, s_warp);
     if (threadIdx.x < 32) {
-        const uint32_t prefix = lookback(P.win_tiles, tile, agg, (uint32_t)H->epoch, H);
+        const uint32_t prefix = lookback(P.win_tiles, tile, agg, epoch, H);
         if (threadIdx.x == 0) {
             s_prefix = prefix;
             if ((int64_t)tile == n_tiles - 1) H->n_win = (int32_t)(prefix + agg);
@@ -865,9 +866,18 @@ __device__ __forceinline__ void append_meta(const DevParams& P, kpx_device_heade
                                             int lam, uint32_t iter, const int32_t* va) {
     constexpr int m = Dims<DYN>::m;
     const int slot = P.win_slot[w];
+    const uint32_t su = (uint32_t)slot;  // < 2^32, as in LaneRollout::start
+    const uint32_t j = su / (uint32_t)lam;
+    const int s = (int)(su - j * (uint32_t)lam);
+    // loads that depend on the slot together, then those that depend on the
+    // region: a winner's chain of round trips to L2 bounds this kernel
     const int r = P.slot_region[slot];
+    const int node = va[min(j, (uint32_t)P.va_cap - 1u)];
+    const int rc = min(max(r, 0), P.R - 1);
+    const uint64_t rk = P.region_key[rc];
+    const int old = P.region_owner[rc];
     // the mapped region must hold this slot's key (a stale entry would not)
-    if (r < 0 || r >= P.R || (uint32_t)P.region_key[r] != (uint32_t)P.N + (uint32_t)slot) {
+    if (r != rc || (uint32_t)rk != (uint32_t)P.N + (uint32_t)slot) {
         set_status(H, KPX_E_INTERNAL);
         H->err_info[1] = (uint32_t)slot;
         return;
@@ -876,10 +886,7 @@ __device__ __forceinline__ void append_meta(const DevParams& P, kpx_device_heade
         P.region_key[r] = P.region_snap[r];
         return;
     }
-    const uint32_t su = (uint32_t)slot;  // < 2^32, as in LaneRollout::start
-    const int j = (int)(su / (uint32_t)lam);
-    const int s = (int)(su - (uint32_t)j * (uint32_t)lam);
-    const int node = va[j];
+    const uint8_t old_set = old >= 0 ? P.set[old] : 0;
     float u[m];
     int K;
     sample_control<m>(P, iter, (uint32_t)node, (uint32_t)s, u, K);
@@ -888,14 +895,13 @@ __device__ __forceinline__ void append_meta(const DevParams& P, kpx_device_heade
     for (int d = 0; d < m; ++d) P.u[(int64_t)d * P.N + id] = u[d];
     P.K[id] = (uint16_t)K;
     P.parent[id] = node;
-    const uint64_t k = pack_key(key_cost(P.region_key[r]), (uint32_t)id);
+    const uint64_t k = pack_key(key_cost(rk), (uint32_t)id);
     P.key[id] = k;
     P.region[id] = r;
     P.set[id] = SET_A;
     P.icount[id] = 0;
-    const int old = P.region_owner[r];
     P.region_key[r] = k;
-    if (old >= 0) P.set[old] = (uint8_t)(P.set[old] | SET_DOM);  // one winner per region: the only writer
+    if (old >= 0) P.set[old] = (uint8_t)(old_set | SET_DOM);  // one winner per region: the only writer
     P.region_owner[r] = id;
 }
 
@@ -981,7 +987,11 @@ __device__ __forceinline__ void stage_tile(const DevParams& P, int tile0, int n_
 constexpr int PRUNE_ROUND_WARPS = PRUNE_TILE / 32;
 static_assert(PRUNE_ROUND_WARPS <= 32, "one warp scans the (round, warp) counts");
 
-template <int THREADS = PRUNE_THREADS>
+// FAR: a walk beyond the tile reads a node's three words together, one round
+// trip to L2 a node instead of up to three (the airplane's 90,000-node trees
+// among 30 columns: 3.88 -> 3.84 ms a call).  The fused kernel's small trees
+// leave their tile too rarely to gain, and the longer loop costs it 0.6 %.
+template <int THREADS = PRUNE_THREADS, bool FAR = true>
 __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header* H, uint32_t tile, int n_tiles,
                                            int n_old, int total, uint32_t epoch, int32_t* va_next,
                                            int32_t* s_parent, uint8_t* s_set, uint8_t* s_icount,
@@ -1032,12 +1042,24 @@ __device__ __forceinline__ void prune_tile(const DevParams& P, kpx_device_header
                     }
                     p = s_parent[p - tile0];
                 }
-                for (; !anc && p >= 0; p = P.parent[p]) {
-                    const uint8_t sp = *(volatile const uint8_t*)&P.set[p];
-                    if (sp & (SET_DOM | SET_ANC)) {
-                        anc = true;
-                    } else if (*(volatile const uint32_t*)&P.clean[p] == epoch) {
-                        break;  // p's strict ancestors are clean, and p is not dominated
+                if constexpr (FAR) {
+                    int32_t up;
+                    for (; !anc && p >= 0; p = up) {
+                        const uint8_t sp = *(volatile const uint8_t*)&P.set[p];
+                        const uint32_t cl = *(volatile const uint32_t*)&P.clean[p];
+                        up = *(volatile const int32_t*)&P.parent[p];
+                        if (sp & (SET_DOM | SET_ANC))
+                            anc = true;
+                        else if (cl == epoch)
+                            break;  // p's strict ancestors are clean, and p is not dominated
+                    }
+                } else {
+                    for (; !anc && p >= 0; p = P.parent[p]) {
+                        const uint8_t sp = *(volatile const uint8_t*)&P.set[p];
+                        if (sp & (SET_DOM | SET_ANC))
+                            anc = true;
+                        else if (*(volatile const uint32_t*)&P.clean[p] == epoch)
+                            break;
                     }
                 }
                 if (!anc) P.clean[i] = epoch;
