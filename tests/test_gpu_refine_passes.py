@@ -70,6 +70,31 @@ def test_batch_equals_its_trajectories_alone(count, steps, n_boxes, aniso):
             assert np.abs(g[i, :n].cpu().numpy() - g64).max() <= 2e-3 * np.abs(g64).max(), i
 
 
+@pytest.mark.parametrize("eps", [-1e-3, -1e-20, 0.0, 1e-40, 1e-30, 1e-20, 8e-16, 9e-16, 1e-15, 1e-7, 1e-3])
+@pytest.mark.parametrize("far_box", [False, True])
+def test_distance_near_a_face(eps, far_box):
+    """A hovering point at x = eps beside a box's face at x = 0 (the hover
+    keeps x exactly), around the distance where the root changes its form, on
+    the face and inside; far_box: with boxes at infinite squared distance in
+    the same list (they begin in the cell of the point, which is that large).
+    Against the FP64 oracle."""
+    prob = scenes.quad_scene(0, clutter=-1)
+    x0 = np.zeros((1, 12), np.float32)
+    x0[0, :3] = [eps, 0.5, 0.5]
+    u = np.zeros((1, 3, 4), np.float32)
+    u[:, :, 0] = prob.param[0] * prob.param[1]
+    k = np.full((1, 3), 7, np.int32)
+    obs = np.float32([[-0.2, 0.2, 0.2, 0.0, 0.8, 0.8], [-0.1, 0.4, 0.4, 0.0, 0.6, 0.6]])
+    if far_box:
+        far = np.float32([[1e23, 0, 0, 1e25, 1, 1]])
+        obs = np.concatenate([far, obs[:1], far, far, obs[1:], far])
+    J, g = refine.evaluate(refine.Batch(prob, x0, u, k, np.int32([3]), obstacles=obs), SPEC, grad=True)
+    J64, g64 = oracle.refine_grad(prob, SPEC, x0[0].astype(np.float64), u[0].astype(np.float64), k[0],
+                                  obstacles=obs.astype(np.float64))
+    assert abs(float(J[0]) - J64) <= 1e-4 * abs(J64)
+    assert np.abs(g[0].cpu().numpy() - g64).max() <= 2e-3 * np.abs(g64).max()
+
+
 def test_segments_without_steps_drop_out():
     """A sequence with empty segments in between (more than a window of 32 of
     them) is the sequence without them."""
