@@ -98,19 +98,13 @@ __global__ void k_b_snapshot(BatchParams BP) {
         P.region_snap[r] = P.region_key[r];
 }
 
-// As PropShape, with one block fewer for the quadcopter: the problem's
-// parameters come from memory here, not from the constant bank, and at 72
-// registers the kernel spills 328 bytes (2,167 us an iteration of 48 mixed
-// problems; 2,110 at 80 registers, 2,190 at 96).
-template <int DYN>
-struct BatchPropShape {
-    static constexpr int threads = PropShape<DYN>::threads;
-    static constexpr int blocks = DYN == KPX_QUAD12 ? 6 : PropShape<DYN>::blocks;
-};
-
-// propagate over the chunks of the class's problems [lo, hi)
+// propagate over the chunks of the class's problems [lo, hi), in PropShape's
+// blocks.  The problem's parameters come from memory here, not from the
+// constant bank; since the stage sums of quad_fma() seven blocks of 128 threads
+// an SM serve the quadcopter here too (an iteration of 48 mixed problems 2.50
+// ms; six 2.57, five 2.66, eight 2.55).
 template <int DYN, int INTEG>
-__global__ void __launch_bounds__(BatchPropShape<DYN>::threads, BatchPropShape<DYN>::blocks) k_b_propagate(BatchParams BP) {
+__global__ void __launch_bounds__(PropShape<DYN>::threads, PropShape<DYN>::blocks) k_b_propagate(BatchParams BP) {
     const int64_t c_lo = BP.chunk_prefix[BP.lo], c_hi = BP.chunk_prefix[BP.hi];
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     int64_t chunk = c_lo + (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -275,11 +269,11 @@ cudaError_t launch_b_propagate_t(const BatchParams& BP, int bps, cudaStream_t s)
     static int per_sm = 0;
     if (!per_sm) {
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_b_propagate<DYN, INTEG>, BatchPropShape<DYN>::threads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_b_propagate<DYN, INTEG>, PropShape<DYN>::threads, 0);
         per_sm = v < 1 ? 1 : v;
     }
     const int use = bps > 0 && bps < per_sm ? bps : per_sm;
-    k_b_propagate<DYN, INTEG><<<b_sm_count() * use, BatchPropShape<DYN>::threads, 0, s>>>(BP);
+    k_b_propagate<DYN, INTEG><<<b_sm_count() * use, PropShape<DYN>::threads, 0, s>>>(BP);
     return cudaGetLastError();
 }
 
