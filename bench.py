@@ -472,9 +472,9 @@ def run_kpx(args):
     value = valid_all / (ms_max / 1e3)
 
     # launches of one step (kpx_graph_info): one graph launch per kpx_iterate
-    # call, holding 1 fused launch plus 7 kernel launches per iteration the
-    # fused kernel left to the loop (begin, propagate, mark, scan, stage, append,
-    # prune); 7 per iteration without the fused kernel
+    # call, holding 1 fused launch (2 but for the quadcopter) plus 7 kernel
+    # launches per iteration the fused kernels left to the loop (begin,
+    # propagate, mark, scan, stage, append, prune); 7 per iteration without them
     max_g, fused = pl.graph_info()
     plan = kpx.Planner.launch_plan(iters, max_g) if max_g else [1] * iters
     pl.reset()
@@ -483,7 +483,8 @@ def run_kpx(args):
     fused_iters = int(pl.header().fused_iterations)
     graph_launches = len(plan) if max_g else 0
     if fused:
-        launches_per_step = 1 + len(plan) + 7 * (iters - fused_iters)  # k_init (reset) first
+        forms = 1 if prob.dyn == scenes.QUAD12 else 2
+        launches_per_step = 1 + forms * len(plan) + 7 * (iters - fused_iters)  # k_init (reset) first
     else:
         launches_per_step = 1 + 7 * iters
 

@@ -127,7 +127,7 @@ enum {
     KPX_FLAG_EARLY_REJECT = 1,
     /* Never run whole iterations in the single-launch cluster kernel (used
      * while an iteration has at most a few thousand slots); every iteration
-     * then launches the eight phase kernels.  Results are identical. */
+     * then launches the phase kernels.  Results are identical. */
     KPX_FLAG_NO_FUSED = 2,
     /* Roll the propagate kernel's slots out in index order instead of in
      * ascending order key (the step count K; the 12D quadcopter's predicted
@@ -259,14 +259,15 @@ kpx_status kpx_set_regions(kpx_planner* p, int32_t n_axes, const kpx_region_axis
  * every iteration is eight plain launches).  The graph's first node writes
  * n into the header's graph_pending.  *fused = 1 when a fused
  * single-launch kernel follows: it runs iterations in one thread-block
- * cluster while an iteration has at most one 32-slot chunk per warp of the
- * cluster and the tree at most 32,768 nodes, and leaves the iterations it
- * did not run in graph_pending.  A loop (a WHILE conditional node) then runs
+ * cluster while an iteration has at most one slot per thread of the cluster
+ * and the tree at most 32,768 nodes, and leaves the iterations it did not run
+ * in graph_pending (the double integrator and the airplane: two such kernels,
+ * the first for up to 512 slots).  A loop (a WHILE conditional node) then runs
  * seven phase kernels once per iteration left (the last block of the last
  * two counts it off graph_pending), until that is 0.  A launch of n
- * iterations thus starts 1 + 7 m kernels, m = the iterations the fused
- * kernel left (the header's fused_iterations counts the ones it ran);
- * without the fused kernel, 7 n. */
+ * iterations thus starts 1 + 7 m kernels (2 + 7 m with two), m = the
+ * iterations the fused kernels left (the header's fused_iterations counts the
+ * ones they ran); without the fused kernel, 7 n. */
 kpx_status kpx_graph_info(kpx_planner* p, int32_t* max_iterations_per_launch, int32_t* fused);
 
 /* Waits for the planner's stream and releases the host handle; the device
@@ -431,8 +432,9 @@ size_t kpx_refine_workspace_size(int32_t count, int32_t max_total_steps);
  * (count, max_total_steps) bytes with a gradient; without one it may be NULL,
  * or >= kpx_refine_workspace_size(0, 0) bytes for the box grid).
  * The box grid: every call that has it builds, on the device, a uniform
- * 16^3 grid over the boxes grown by the distance beyond which a box's term
- * is dropped, each cell listing in index order the boxes that can reach it;
+ * grid (32^3, or 16^3 when the finer lists would not fit the workspace) over
+ * the boxes grown by the distance beyond which a box's term is dropped, each
+ * cell listing in index order the boxes that can reach it;
  * a point then tests only its cell's boxes.  The terms kept are the same as
  * with every box tested; the summation order differs, so results equal those
  * of a call without the grid up to FP32 rounding, and calls with the grid
@@ -513,7 +515,7 @@ typedef struct {
     uint64_t total_candidates, total_valid, total_winners;
     uint64_t t_start_ns, t_first_solution_ns, t_last_ns;
     int32_t traj_len;
-    int32_t graph_ctl;         /* internal: the fused iteration's control word */
+    int32_t graph_ctl;         /* internal: the fused iteration's control word; finished blocks of the loop's */
     uint64_t total_steps;      /* integration steps executed by Propagate since create/reset */
     uint64_t total_box_tests;  /* point-in-box tests executed by Propagate since create/reset */
     uint32_t err_info[4];

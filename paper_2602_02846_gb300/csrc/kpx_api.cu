@@ -382,11 +382,13 @@ cudaMemsetParams count_params(const kpx_planner* p, int n) {
 //   count node (memset: graph_pending = n)
 //   -> the fused kernel (kpx_fused.cu), when the device can run its cluster:
 //      iterations while the problem is small; the rest stay in graph_pending
+//      (two of them, the narrow and the wide form, for the double integrator
+//      and the airplane)
 //   -> WHILE node: up to kLoopIterations (kLoopIterationsFused behind the
 //      fused kernel) iterations of the phase kernels per trip, until
 //      graph_pending is 0 (each iteration's last kernel
 //      counts it off).
-// With the fused kernel the loop's handle starts at 0 and the fused kernel
+// With the fused kernel the loop's handle starts at 0 and its last form
 // sets it; without it the handle starts at 1 (n >= 1).  Only the count
 // node changes between launches.
 cudaError_t build_loop_graph(kpx_planner* p, bool fused) {
@@ -402,25 +404,27 @@ cudaError_t build_loop_graph(kpx_planner* p, bool fused) {
         e = cudaGraphAddMemsetNode(&count, g, nullptr, 0, &m);
     }
     dep = count;
-    if (e == cudaSuccess && fused) {
-        e = cudaStreamBeginCaptureToGraph(p->capture_stream, g, &count, nullptr, 1, cudaStreamCaptureModeRelaxed);
+    cudaGraphNode_t chain[3] = {count};  // the nodes so far, each behind the one before
+    const int forms = fused ? (fused_wide_size(p->P) > 0 ? 2 : 1) : 0;
+    for (int f = 0; e == cudaSuccess && f < forms; ++f) {
+        e = cudaStreamBeginCaptureToGraph(p->capture_stream, g, &dep, nullptr, 1, cudaStreamCaptureModeRelaxed);
         if (e == cudaSuccess) {
-            le = launch_fused(p->P, -1, h, 1, p->capture_stream);
+            le = launch_fused(p->P, f == 1, -1, h, f == forms - 1, p->capture_stream);
             cudaGraph_t out = nullptr;
             e = cudaStreamEndCapture(p->capture_stream, &out);
             if (le != cudaSuccess) e = le;
         }
-        // the captured fused kernel: the graph's only kernel node
-        cudaGraphNode_t nodes[2] = {};
-        size_t n_nodes = 2;
+        // the captured kernel: the graph's one new node
+        cudaGraphNode_t nodes[3] = {};
+        size_t n_nodes = 3;
         if (e == cudaSuccess) e = cudaGraphGetNodes(g, nodes, &n_nodes);
-        if (e == cudaSuccess && n_nodes != 2) e = cudaErrorUnknown;
+        if (e == cudaSuccess && n_nodes != (size_t)(f + 2)) e = cudaErrorUnknown;
         for (size_t k = 0; e == cudaSuccess && k < n_nodes; ++k) {
-            cudaGraphNodeType t;
-            e = cudaGraphNodeGetType(nodes[k], &t);
-            if (e == cudaSuccess && t == cudaGraphNodeTypeKernel) dep = nodes[k];
+            bool seen = false;
+            for (int c = 0; c <= f; ++c) seen |= nodes[k] == chain[c];
+            if (!seen) dep = chain[f + 1] = nodes[k];
         }
-        if (e == cudaSuccess && dep == count) e = cudaErrorUnknown;
+        if (e == cudaSuccess && !chain[f + 1]) e = cudaErrorUnknown;
     }
     cudaGraphNodeParams cp = {};
     if (e == cudaSuccess) {
@@ -1490,8 +1494,9 @@ extern "C" kpx_status kpx_plan_static(const kpx_dynamics* dyn, const kpx_workspa
     };
     int32_t left = n_iters;
     if (e == cudaSuccess && left > 0 && !(P.flags & KPX_FLAG_NO_FUSED) && fused_cluster_size(P) > 0 &&
-        launch_fused(P, left, 0, 0, pl.stream) == cudaSuccess) {
-        e = sync_header();
+        launch_fused(P, false, left, 0, 0, pl.stream) == cudaSuccess) {
+        if (fused_wide_size(P) > 0) e = launch_fused(P, true, -1, 0, 0, pl.stream);
+        if (e == cudaSuccess) e = sync_header();
         left = e == cudaSuccess ? h.graph_pending : 0;
     }
     cudaGetLastError();  // an unavailable cluster launch leaves every iteration to the phase kernels

@@ -34,19 +34,28 @@ namespace kpx {
 
 namespace {
 
-// Threads of a CTA.  The double integrator and the airplane, whose checks cost
-// several integrations each, split a rollout over lanes of several warps when
-// the slots leave some idle (roll_part): 512 threads on 16 SMs hold 2,048
-// rollouts in four parts, 4,096 in two, or 8,192 whole.  Eight parts cost more
-// unchecked steps than they save checks (200 iterations of 576 slots: 2.04 ms
-// against 1.83 ms in four).  The rollouts bound these iterations: 200 of the airplane among 300 boxes, 2,944 slots each,
-// take 2.23 ms; 2.33 ms with 256 threads, 2.32 ms unsplit; 2.36 ms with 256
-// threads unsplit, a step integrated ahead of its checks and a cell's two
-// offsets in two words, as it was.  The quadcopter's integration costs more
-// than its checks and needs the registers: 256 threads, and lanes of one warp
-// share the checks (roll_candidate_coop).
-template <int DYN>
-constexpr int FUSED_THREADS = DYN == KPX_QUAD12 ? 256 : 512;
+// The double integrator and the airplane have two forms of this kernel, one
+// launched behind the other.  The narrow one (256 threads a CTA; the
+// quadcopter's only form) takes iterations of up to FUSED_NARROW_SLOTS slots
+// and shares a rollout among lanes of a warp (roll_candidate_coop).  The wide
+// one (512 threads) splits a rollout over lanes of several warps when the slots
+// leave some idle (roll_part), since their checks cost several integrations
+// each: 16 SMs hold 2,048 rollouts in four parts, 4,096 in two, or 8,192 whole.
+// The rollouts bound the wide form's iterations: 200 of the airplane among 300
+// boxes, 2,944 slots each, take 2.23 ms; 2.33 ms with 256 threads, 2.32 ms
+// unsplit; 2.36 ms with 256 threads unsplit, a step integrated ahead of its
+// checks and a cell's two offsets in two words, as it was.  Eight parts cost
+// more unchecked steps than they save checks (200 iterations of 576 slots: 2.04
+// ms against 1.83 ms in four).  Below the line the wide form's barriers and its
+// longest part cost more than the narrow form's shared checks (200 iterations
+// of the airplane at 43, 99, 206 and 485 slots on average: 1.39, 1.51, 1.60 and
+// 1.78 ms with the narrow form in front, 1.74, 1.75, 1.75 and 1.80 ms in the wide
+// one alone; the double integrator at 127: 1.53 and 1.65 ms).  A growing problem
+// pays the second launch, 10 of 640 us in the double integrator's room.  The
+// quadcopter's integration costs more than its checks and needs the registers.
+constexpr int FUSED_NARROW_SLOTS = 512;
+template <int DYN, bool WIDE>
+constexpr int FUSED_THREADS = WIDE ? 512 : 256;
 constexpr int FUSED_MAX_PARTS = 4;
 constexpr int FUSED_MAX_CLUSTER = 16;
 constexpr int FUSED_MAX_NODES = 32768;
@@ -158,11 +167,10 @@ __device__ __forceinline__ void fused_begin(const DevParams& P, kpx_device_heade
     H->graph_ctl = ctl;
 }
 
-template <int DYN, int INTEG>
-__global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
+template <int DYN, int INTEG, bool WIDE>
+__global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
     k_fused(DevParams P, int n_iter, cudaGraphConditionalHandle handle, int use_handle, int grid_smem) {
-    constexpr int THREADS = FUSED_THREADS<DYN>, WARPS = THREADS / 32;
-    constexpr bool SPLIT = DYN != KPX_QUAD12;
+    constexpr int THREADS = FUSED_THREADS<DYN, WIDE>, WARPS = THREADS / 32;
     extern __shared__ __align__(16) unsigned char fused_grid[];
     __shared__ uint32_t s_prefix;
     __shared__ int32_t s_parent[PRUNE_TILE];
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     __shared__ uint8_t s_icount[PRUNE_TILE];
     __shared__ uint32_t s_counts[PRUNE_ROUND_WARPS];
     __shared__ uint32_t s_cnt[FUSED_MAX_CLUSTER * WARPS];  // winners per chunk (every CTA's copy)
-    __shared__ uint2 s_part[SPLIT ? THREADS : 1];  // a split rollout's parts: steps (top bit: all valid), box tests
+    __shared__ uint2 s_part[WIDE ? THREADS : 1];  // a split rollout's parts: steps (top bit: all valid), box tests
     // While the launch runs, the header lives in CTA 0's shared memory: the
     // leader's bookkeeping stays on the SM, and the few header updates of
     // other CTAs (a status, the goal key) reach it over distributed shared
@@ -183,6 +191,10 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     __shared__ __align__(16) IterParams s_it;  // this CTA's copy of the iteration's parameters
     constexpr int HDR_WORDS = (int)(sizeof(kpx_device_header) / sizeof(uint32_t));
     static_assert(sizeof(kpx_device_header) % sizeof(uint32_t) == 0, "header size");
+    if (WIDE && P.hdr->graph_pending <= 0) {  // the narrow form left nothing (every CTA reads the same)
+        if (blockIdx.x == 0 && threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, 0u);
+        return;
+    }
     if (blockIdx.x == 0) {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(P.hdr);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&s_hdr);
@@ -195,6 +207,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     const int n_cta = (int)gridDim.x;  // the grid is one cluster
     const int64_t gtid = (int64_t)blockIdx.x * THREADS + threadIdx.x;
     const int64_t gthreads = (int64_t)n_cta * THREADS;
+    const int64_t max_slots = WIDE || DYN == KPX_QUAD12 ? gthreads : min(gthreads, (int64_t)FUSED_NARROW_SLOTS);
     const bool early = (P.flags & KPX_FLAG_EARLY_REJECT) != 0;
     GridView G{P.cell_start, P.cell_box};
     if (grid_smem) {  // the obstacle grid is read-only while planning
@@ -213,7 +226,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     // the leader's warp keeps the books through CTA 0's own window
     kpx_device_header* HL = &s_hdr;
     if (lead_warp) {
-        if (leader) fused_begin(P, HL, n_iter, gthreads);
+        if (leader) fused_begin(P, HL, n_iter, max_slots);
         publish_iteration(HL, &s_it, n_cta);
     }
     int done = 0;
@@ -245,12 +258,12 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
         }
         // propagate (Alg. 2): chunks of slots, warp-major across the CTAs.
         // When the slots leave threads idle, a rollout is split over lanes of
-        // `parts` warps (roll_part), a chunk being 32 slots; or (the
-        // quadcopter) g lanes of a warp share it, a chunk being 32 / g slots.
+        // `parts` warps (roll_part; the wide form), a chunk being 32 slots; or
+        // g lanes of a warp share it, a chunk being 32 / g slots.
         // The lane that keeps a candidate holds it in registers.
-        const int g = SPLIT || early ? 1 : coop_lanes(n_slots, gthreads);
+        const int g = WIDE || early ? 1 : coop_lanes(n_slots, gthreads);
         int parts = 1;
-        if (SPLIT && !early)
+        if (WIDE && !early)
             while (parts < FUSED_MAX_PARTS && n_slots * (2 * parts) <= gthreads) parts *= 2;
         const int warp = threadIdx.x >> 5;
         const int n_chunks = n_cta * (WARPS / parts);
@@ -262,7 +275,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
         {
             uint32_t steps = 0, tests = 0, n_valid = 0;
             const bool live = slot < n_slots;
-            if (SPLIT && parts > 1) {
+            if (WIDE && parts > 1) {
                 bool ok = false;
                 if (live) {
                     C.R.start(P, va, lam, iter, slot);
@@ -296,7 +309,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
                         roll_candidate<DYN, INTEG, true>(P, G, lam, iter, va, true, slot, C, steps, tests);
                     else
                         roll_candidate<DYN, INTEG, false>(P, G, lam, iter, va, true, slot, C, steps, tests);
-                } else if (SPLIT) {  // 16 warps: nothing to overlap
+                } else if (WIDE || DYN == KPX_DI6) {  // 16 warps, or a short step: nothing to overlap
                     if (grid_smem)
                         roll_candidate<DYN, INTEG, true>(P, G, lam, iter, va, false, slot, C, steps, tests);
                     else
@@ -381,7 +394,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
             if (leader) {
                 end_counters(P, HL, false);
                 HL->fused_iterations += 1;
-                fused_begin(P, HL, n_iter - done, gthreads);
+                fused_begin(P, HL, n_iter - done, max_slots);
             }
             publish_iteration(HL, &s_it, n_cta);
         }
@@ -390,7 +403,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
             if (leader) {
                 end_counters(P, HL, false);
                 HL->fused_iterations += 1;
-                fused_begin(P, HL, n_iter - done, gthreads);
+                fused_begin(P, HL, n_iter - done, max_slots);
             }
             publish_iteration(HL, &s_it, n_cta);
         }
@@ -410,26 +423,26 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN>, 1)
     }
 }
 
-template <int DYN, int INTEG>
-int fused_cluster_size_t(const DevParams&, int) {
+template <int DYN, int INTEG, bool WIDE>
+int form_cluster_size() {
     static int size = -1;
     if (size < 0) {
         size = 0;
-        if (cudaFuncSetAttribute(k_fused<DYN, INTEG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
             cudaSuccess) {
             cudaGetLastError();
         }
-        if (cudaFuncSetAttribute(k_fused<DYN, INTEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)FUSED_GRID_SMEM_MAX) != cudaSuccess) {
             cudaGetLastError();
             return size;  // 0: unavailable
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(FUSED_MAX_CLUSTER);
-        cfg.blockDim = dim3(FUSED_THREADS<DYN>);
+        cfg.blockDim = dim3(FUSED_THREADS<DYN, WIDE>);
         cfg.dynamicSmemBytes = FUSED_GRID_SMEM_MAX;  // the cluster must fit with a staged grid
         int cl = 0;
-        if (cudaOccupancyMaxPotentialClusterSize(&cl, (const void*)k_fused<DYN, INTEG>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxPotentialClusterSize(&cl, (const void*)k_fused<DYN, INTEG, WIDE>, &cfg) != cudaSuccess) {
             cudaGetLastError();
             cl = 0;
         }
@@ -442,15 +455,29 @@ int fused_cluster_size_t(const DevParams&, int) {
 }
 
 template <int DYN, int INTEG>
-cudaError_t launch_fused_t(const DevParams& P, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
-                           cudaStream_t s) {
-    const int cl = fused_cluster_size_t<DYN, INTEG>(P, 0);
+int fused_cluster_size_t(const DevParams&, int) {
+    return form_cluster_size<DYN, INTEG, false>();
+}
+
+// the wide form's cluster: 0 when the system has none
+template <int DYN, int INTEG>
+int fused_wide_size_t(const DevParams&, int) {
+    if constexpr (DYN == KPX_QUAD12)
+        return 0;
+    else
+        return form_cluster_size<DYN, INTEG, true>();
+}
+
+template <int DYN, int INTEG, bool WIDE>
+cudaError_t launch_form(const DevParams& P, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+                        cudaStream_t s) {
+    const int cl = form_cluster_size<DYN, INTEG, WIDE>();
     if (cl == 0) return cudaErrorNotSupported;
     const size_t grid_bytes = grid_start_bytes(P.n_cells) + (size_t)P.grid_entries * 2 * sizeof(float4);
     const int grid_smem = P.n_obs > 0 && grid_bytes <= FUSED_GRID_SMEM_MAX ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(FUSED_THREADS<DYN>);
+    cfg.blockDim = dim3(FUSED_THREADS<DYN, WIDE>);
     cfg.dynamicSmemBytes = grid_smem ? grid_bytes : 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -460,7 +487,15 @@ cudaError_t launch_fused_t(const DevParams& P, int n_iter, cudaGraphConditionalH
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_fused<DYN, INTEG>, P, n_iter, handle, use_handle, grid_smem);
+    return cudaLaunchKernelEx(&cfg, k_fused<DYN, INTEG, WIDE>, P, n_iter, handle, use_handle, grid_smem);
+}
+
+template <int DYN, int INTEG>
+cudaError_t launch_fused_t(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle,
+                           int use_handle, cudaStream_t s) {
+    if constexpr (DYN != KPX_QUAD12)
+        if (wide) return launch_form<DYN, INTEG, true>(P, n_iter, handle, use_handle, s);
+    return wide ? cudaErrorInvalidValue : launch_form<DYN, INTEG, false>(P, n_iter, handle, use_handle, s);
 }
 
 #define KPX_FUSED_DISPATCH(FN, P, ...)                                                   \
@@ -481,9 +516,14 @@ int fused_cluster_size(const DevParams& P) {
     return 0;
 }
 
-cudaError_t launch_fused(const DevParams& P, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+int fused_wide_size(const DevParams& P) {
+    KPX_FUSED_DISPATCH(fused_wide_size_t, P, 0);
+    return 0;
+}
+
+cudaError_t launch_fused(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
                          cudaStream_t s) {
-    KPX_FUSED_DISPATCH(launch_fused_t, P, n_iter, handle, use_handle, s);
+    KPX_FUSED_DISPATCH(launch_fused_t, P, wide, n_iter, handle, use_handle, s);
     return cudaErrorInvalidValue;
 }
 

@@ -298,11 +298,14 @@ void prepare_launches(const DevParams& P);
 // fused iterations (kpx_fused.cu): CTAs of the single cluster that runs
 // them for this problem's dynamics (0: unavailable on this device)
 int fused_cluster_size(const DevParams& P);
+// CTAs of the wide form's cluster (0: the system has none, or unavailable); it
+// goes behind the narrow one, with n_iter < 0
+int fused_wide_size(const DevParams& P);
 // up to n_iter iterations in one launch while the problem stays small
 // (n_iter < 0: the count the header's graph_pending holds at launch); the
 // rest go to the phase kernels through graph_pending and, when use_handle,
 // the graph's conditional handle (1: phase kernels needed)
-cudaError_t launch_fused(const DevParams& P, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+cudaError_t launch_fused(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
                          cudaStream_t s);
 
 // trajectory refinement (kpx_adjoint.cu: objective, adjoint gradient and

@@ -15,7 +15,7 @@
 //              the graphs)
 //   prune      PruneNodes (Alg. 3) over the pre-append tree, fused with the
 //              compaction of the next V_A list (Alg. 5)
-//   end        counters
+//   end        counters (in the graphs: the last block of stage and prune)
 #include <cuda_runtime.h>
 
 #include "kpx_phases.cuh"

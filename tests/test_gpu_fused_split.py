@@ -1,6 +1,6 @@
-"""The one-cluster kernel's split of a rollout over several warps: at slot
-counts around each number of parts' limit (and one slot, one warp, and the
-largest iteration the kernel takes), with the obstacle grid absent, copied into
+"""The one-cluster kernel's two forms and the wide one's split of a rollout
+over several warps: at slot counts around the line between them and each number
+of parts' limit (and one slot, one warp, and the largest iteration taken), with the obstacle grid absent, copied into
 shared memory and too large for that, against the phase kernels, bit for bit."""
 import numpy as np
 import pytest
@@ -12,7 +12,7 @@ import paper_2602_02846_gb300 as kpx  # noqa: E402
 from paper_2602_02846_gb300 import scenes  # noqa: E402
 from tests.test_gpu_fused import _same, _state  # noqa: E402
 
-SLOTS = [1, 31, 33, 1023, 1024, 1025, 2048, 2049, 4096, 4097, 8191, 8192, 8193]
+SLOTS = [1, 31, 33, 511, 512, 513, 1023, 1024, 1025, 2048, 2049, 4096, 4097, 8191, 8192, 8193]
 
 
 @pytest.fixture(scope="module", autouse=True)
