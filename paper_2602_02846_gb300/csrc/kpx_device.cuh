@@ -343,6 +343,11 @@ __device__ __forceinline__ void cell_range_ws(const DevParams& P, const GridView
 template <bool SMEM>
 __device__ __forceinline__ bool walk_cell(const GridView& G, float px, float py, float pz, int e0, int e1,
                                           uint32_t& tests) {
+    // most cells are empty: a test of its own, and no unrolled walk behind it
+    // (the quadcopter's propagate in the building 0.232 -> 0.228 ms; from
+    // shared memory the loop's own test is as fast)
+    if (!SMEM && e0 >= e1) return false;
+#pragma unroll 1
     for (int e = e0; e < e1; ++e) {
         const float4 lo = grid_ld<SMEM>(G.cell_box + 2 * e);
         const float4 hi = grid_ld<SMEM>(G.cell_box + 2 * e + 1);
