@@ -670,7 +670,8 @@ __device__ __forceinline__ int64_t propagate_unit_chunk(int64_t q, int64_t n_slo
 // registers.  Seven blocks of 128 threads at 72 registers (28 warps an SM) beat
 // three of 256 at 80 (24 warps): 0.249 against 0.256 ms a launch in the
 // building; eight at 64 registers, with spills, take 0.251, six 0.255, two of
-// 256 0.277 (0.234 since, with the stage sums of quad_fma()).
+// 256 0.277 (0.228 since, with the stage sums of quad_fma() and the walk of
+// walk_cell()).
 template <int DYN>
 struct PropShape {
     static constexpr int threads = DYN == KPX_QUAD12 ? 128 : 256;
