@@ -4,7 +4,8 @@ nvcc cross-compiles without a GPU; the translation units compile in parallel.
 FP contraction is off (-fmad=false) in every unit that runs the planner's
 arithmetic: fused multiply-adds appear only where the kernels write fmaf(),
 which keeps re-materialised rollouts bit-identical.  The refinement gradient
-kernels (kpx_adjoint.cu) contract freely.
+kernels (kpx_adjoint.cu) may contract: there the box terms are left to the
+compiler, and the dynamics and the adjoint write their roundings out.
 """
 from __future__ import annotations
 
@@ -24,8 +25,8 @@ SOURCES = ["kpx_kernels.cu", "kpx_fused.cu", "kpx_batch.cu", "kpx_adjoint.cu", "
            "kpx_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off", "-I", INCLUDE, "-I", CSRC]
-# the refinement gradient kernels reproduce nothing bit for bit, so they may
-# contract into FMAs; every other unit keeps the planner's arithmetic
+# the refinement gradient kernels need not reproduce the planner's arithmetic,
+# so they may contract into FMAs; every other unit keeps it
 FMAD = {"kpx_adjoint.cu": "-fmad=true", "kpx_peak.cu": "-fmad=true"}
 
 
