@@ -448,13 +448,11 @@ extern "C" kpx_status kpx_refine_validate(const kpx_dynamics* dyn, const kpx_wor
     const int row = per_block | 1;
     const size_t boxes = (size_t)8 * n_obstacles * sizeof(float);
     size_t smem = (size_t)VAL_ROW_BYTES * row + VAL_GRID_BYTES;
-    const bool smem_boxes = smem + boxes <= 226 * 1024;
+    const bool smem_boxes = smem + boxes <= REFINE_SMEM_MAX;
     if (smem_boxes) smem += boxes;
     const auto kernel = P.iso_inertia ? (smem_boxes ? k_refine_validate<true, true> : k_refine_validate<true, false>)
                                       : (smem_boxes ? k_refine_validate<false, true> : k_refine_validate<false, false>);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return KPX_E_CUDA;
+    if (allow_smem((const void*)kernel, smem) != cudaSuccess) return KPX_E_CUDA;
     kernel<<<(count + per_block - 1) / per_block, VAL_WARPS * 32, smem, reinterpret_cast<cudaStream_t>(cuda_stream)>>>(
         P, V, per_block, row);
     return cudaGetLastError() == cudaSuccess ? KPX_OK : KPX_E_CUDA;

@@ -62,6 +62,18 @@ __device__ __forceinline__ void feed_steps(const Params& R, int64_t tr, int S, i
     }
 }
 
+// Dynamic shared memory that a refinement kernel may be launched with: the
+// 227 KB of a block less 1 KB for the kernels' static arrays.  The limit belongs
+// to the function, not to the launch, so every caller sets this same value: one
+// that set its own call's size could lower it under another thread's launch.
+constexpr size_t REFINE_SMEM_MAX = 226 * 1024;
+
+inline cudaError_t allow_smem(const void* fn, size_t bytes) {
+    if (bytes > REFINE_SMEM_MAX) return cudaErrorInvalidValue;
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REFINE_SMEM_MAX);
+}
+
 inline int device_sms() {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
