@@ -37,11 +37,15 @@ struct ValidateParams {
 // sixteen warps lay out the controls of the next 32 steps and check the states
 // of the previous ones (a trajectory a warp, a step a lane): bounds, then the
 // boxes of the point's cell in a grid that the block builds over the workspace
-// box.  The first state that fails ends its trajectory.  One more warp adds
-// the FP64 costs.  Bound: the longest trajectory's chain of RK4 steps, about
-// 400 cycles each.  With a warp per trajectory, every step waiting for its
-// 1,000 box tests (31 a lane), 512 sequences of up to 2,076 steps took 6.03
-// ms; this form takes 0.49 ms.
+// box, or every box where the grid would not pay or its lists do not fit.  The
+// first state that fails ends its trajectory.  One more warp adds the FP64
+// costs.  Bound: the longest trajectory's chain of RK4 steps, about 400 cycles
+// each.  With a warp per trajectory, every step waiting for its 1,000 box
+// tests (31 a lane), 512 sequences of up to 2,076 steps took 6.03 ms; this form
+// takes 0.46 ms.  (Calls of a few steps, or among large boxes, took up to 25
+// times a warp's time while every block built a grid, a warp a box and its
+// size known only once it was built: 4,096 boxes over the whole workspace 2.2
+// ms, now 0.05.)
 constexpr int VAL_CHECK_WARPS = 16;
 constexpr int VAL_COST_WARP = 4;  // on one scheduler with the integrating warp 0, which so gets the fewest checkers
 constexpr int VAL_WARPS = VAL_CHECK_WARPS + 2;
@@ -50,6 +54,14 @@ constexpr int VAL_ROW_BYTES = 2 * 32 * (int)(sizeof(float4) + sizeof(int) + 12 *
 constexpr int VAL_AXIS = 16;
 constexpr int VAL_CELLS = VAL_AXIS * VAL_AXIS * VAL_AXIS;
 constexpr int VAL_ENTRIES = 16384;
+// A block builds its grid when its trajectories have more steps than this
+// together.  Both the grid and the tests it saves grow with the boxes: 4,000
+// boxes of 0.02 cost it 22 us (1,000: 5 us), and testing every one of them
+// costs a lone trajectory 0.4 ns a step and box, 32 trajectories of a block 0.1.
+// With 4,000 boxes, grid / every box: one trajectory of 4 steps 67 / 49 us, of
+// 16 72 / 78, of 32 74 / 119; four of 4 steps 71 / 53, of 16 74 / 96; 32 of 1
+// step 73 / 72, of 4 73 / 114.
+constexpr uint32_t VAL_GRID_STEPS = 24;
 constexpr int VAL_GRID_BYTES = VAL_CELLS * (int)sizeof(int) + VAL_ENTRIES * (int)sizeof(uint16_t);
 
 // the integrating and the checking warps, once per 32 steps
@@ -85,38 +97,75 @@ __device__ __forceinline__ void box_of(const ValidateParams& V, const float4* s_
     }
 }
 
-// called by the whole block; a warp per box, its cells over the lanes
+// The cells of box b: first cell and cells an axis (none for b past the boxes).
+struct BoxCells {
+    int x0, y0, z0, nx, ny, n;
+
+    __device__ __forceinline__ int cell(int k) const {
+        return ((z0 + k / (nx * ny)) * VAL_AXIS + y0 + k / nx % ny) * VAL_AXIS + x0 + k % nx;
+    }
+};
+
+template <bool SMEM_BOXES>
+__device__ __forceinline__ BoxCells cells_of(const DevParams& P, const ValidateParams& V, const float4* s_box,
+                                             const ValGrid& G, int b) {
+    BoxCells c = {};
+    if (b >= V.n_obs) return c;
+    float4 lo, hi;
+    box_of<SMEM_BOXES>(V, s_box, b, lo, hi);
+    c.x0 = G.axis_cell(P, lo.x, 0);
+    c.y0 = G.axis_cell(P, lo.y, 1);
+    c.z0 = G.axis_cell(P, lo.z, 2);
+    c.nx = max(G.axis_cell(P, hi.x, 0) - c.x0 + 1, 0);
+    c.ny = max(G.axis_cell(P, hi.y, 1) - c.y0 + 1, 0);
+    c.n = c.nx * c.ny * max(G.axis_cell(P, hi.z, 2) - c.z0 + 1, 0);
+    return c;
+}
+
+// Called by the whole block: a lane a box, and a box of many cells by its
+// whole warp.  The cells are added up first, so lists that do not fit cost
+// nothing more.
 template <bool SMEM_BOXES>
 __device__ void build_grid(const DevParams& P, const ValidateParams& V, const float4* s_box, ValGrid& G) {
-    __shared__ int s_warp[32];
-    __shared__ int s_total;
+    constexpr int THREADS = VAL_WARPS * 32, LANE_CELLS = 16;  // cells that a lane takes alone
+    __shared__ int s_warp[VAL_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float w = P.ws_hi[a] - P.ws_lo[a];
         G.inv[a] = w > 0.0f ? (float)VAL_AXIS / w : 0.0f;
     }
-    for (int c = threadIdx.x; c < VAL_CELLS; c += VAL_WARPS * 32) G.end[c] = 0;
+    int total = 0;
+    for (int b = threadIdx.x; b < V.n_obs; b += THREADS) total += cells_of<SMEM_BOXES>(P, V, s_box, G, b).n;
+    total = __reduce_add_sync(0xFFFFFFFFu, total);
+    if (lane == 0) s_warp[warp] = total;
+    for (int c = threadIdx.x; c < VAL_CELLS; c += THREADS) G.end[c] = 0;
     __syncthreads();
-#pragma unroll
+    total = 0;
+    for (int w = 0; w < VAL_WARPS; ++w) total += s_warp[w];
+    G.ok = total <= VAL_ENTRIES;
+    if (!G.ok) return;
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {  // counts, then lists
-        for (int b = warp; b < V.n_obs; b += VAL_WARPS) {
-            float4 lo, hi;
-            box_of<SMEM_BOXES>(V, s_box, b, lo, hi);
-            const int x0 = G.axis_cell(P, lo.x, 0), y0 = G.axis_cell(P, lo.y, 1), z0 = G.axis_cell(P, lo.z, 2);
-            const int nx = max(G.axis_cell(P, hi.x, 0) - x0 + 1, 0), ny = max(G.axis_cell(P, hi.y, 1) - y0 + 1, 0),
-                      nz = max(G.axis_cell(P, hi.z, 2) - z0 + 1, 0);
-            for (int k = lane; k < nx * ny * nz; k += 32) {
-                const int c = ((z0 + k / (nx * ny)) * VAL_AXIS + y0 + k / nx % ny) * VAL_AXIS + x0 + k % nx;
-                const int pos = atomicAdd(&G.end[c], 1);  // second pass: from the cell's first entry on
-                if (pass == 1) G.ids[pos] = (uint16_t)b;
+        auto visit = [&](int b, int c) {
+            const int pos = atomicAdd(&G.end[c], 1);  // second pass: from the cell's first entry on
+            if (pass == 1) G.ids[pos] = (uint16_t)b;
+        };
+        for (int b0 = warp * 32; b0 < V.n_obs; b0 += THREADS) {
+            const BoxCells m = cells_of<SMEM_BOXES>(P, V, s_box, G, b0 + lane);
+            if (m.n <= LANE_CELLS)
+                for (int k = 0; k < m.n; ++k) visit(b0 + lane, m.cell(k));
+            for (uint32_t many = __ballot_sync(0xFFFFFFFFu, m.n > LANE_CELLS); many; many &= many - 1) {
+                const int b = b0 + __ffs(many) - 1;
+                const BoxCells w = cells_of<SMEM_BOXES>(P, V, s_box, G, b);
+                for (int k = lane; k < w.n; k += 32) visit(b, w.cell(k));
             }
         }
         __syncthreads();
         if (pass == 1) break;
         // counts -> first entries (the second pass moves them to the ends)
         constexpr int PER = VAL_CELLS / 512;
-        static_assert(VAL_WARPS * 32 >= 512, "512 threads scan the cells");
+        static_assert(THREADS >= 512, "512 threads scan the cells");
         int v[PER], sum = 0;
         const bool in = threadIdx.x < 512;
 #pragma unroll
@@ -134,7 +183,6 @@ __device__ void build_grid(const DevParams& P, const ValidateParams& V, const fl
         __syncthreads();
         int run = x - sum;
         for (int w = 0; w < warp; ++w) run += s_warp[w];
-        if (threadIdx.x == VAL_WARPS * 32 - 1) s_total = run + sum;
         if (in) {
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
@@ -143,26 +191,37 @@ __device__ void build_grid(const DevParams& P, const ValidateParams& V, const fl
             }
         }
         __syncthreads();
-        G.ok = s_total <= VAL_ENTRIES;
-        if (!G.ok) return;
     }
 }
 
-// whether a point of the workspace box lies in a box
+// whether a point of the workspace box lies in a box that its cell lists
 template <bool SMEM_BOXES>
-__device__ __forceinline__ bool in_a_box(const DevParams& P, const ValidateParams& V, const float4* s_box,
-                                         const ValGrid& G, float px, float py, float pz) {
-    int e0 = 0, e1 = V.n_obs;
-    if (G.ok) {
-        const int c = (G.axis_cell(P, pz, 2) * VAL_AXIS + G.axis_cell(P, py, 1)) * VAL_AXIS + G.axis_cell(P, px, 0);
-        e0 = c > 0 ? G.end[c - 1] : 0;
-        e1 = G.end[c];
-    }
+__device__ __forceinline__ bool in_a_listed_box(const DevParams& P, const ValidateParams& V, const float4* s_box,
+                                                const ValGrid& G, float px, float py, float pz) {
+    const int c = (G.axis_cell(P, pz, 2) * VAL_AXIS + G.axis_cell(P, py, 1)) * VAL_AXIS + G.axis_cell(P, px, 0);
+    const int e1 = G.end[c];
     bool hit = false;
-    for (int e = e0; e < e1 && !hit; ++e) {
+    for (int e = c > 0 ? G.end[c - 1] : 0; e < e1 && !hit; ++e) {
         float4 lo, hi;
-        box_of<SMEM_BOXES>(V, s_box, G.ok ? (int)G.ids[e] : e, lo, hi);
+        box_of<SMEM_BOXES>(V, s_box, (int)G.ids[e], lo, hi);
         hit = px >= lo.x && px <= hi.x && py >= lo.y && py <= hi.y && pz >= lo.z && pz <= hi.z;
+    }
+    return hit;
+}
+
+// whether a point lies in one of the boxes first, first + stride, ...; four at
+// a time, so that their loads overlap
+template <bool SMEM_BOXES>
+__device__ __forceinline__ bool in_a_box(const ValidateParams& V, const float4* s_box, int first, int stride, float px,
+                                         float py, float pz) {
+    bool hit = false;
+    for (int b = first; b < V.n_obs && !hit; b += 4 * stride) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float4 lo, hi;
+            box_of<SMEM_BOXES>(V, s_box, min(b + k * stride, V.n_obs - 1), lo, hi);
+            hit |= px >= lo.x && px <= hi.x && py >= lo.y && py <= hi.y && pz >= lo.z && pz <= hi.z;
+        }
     }
     return hit;
 }
@@ -205,10 +264,9 @@ __global__ void __launch_bounds__(VAL_WARPS * 32, 1) k_refine_validate(DevParams
         }
     }
     __syncthreads();
-    if (V.n_obs > 0)
-        build_grid<SMEM_BOXES>(P, V, s_box, G);
-    else
-        G.ok = false;
+    G.ok = false;
+    const uint32_t steps = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)min(max(s_total[lane], 0ll), 1ll << 20));
+    if (V.n_obs > 0 && steps > VAL_GRID_STEPS) build_grid<SMEM_BOXES>(P, V, s_box, G);
     const int64_t tr = base + lane;
     if (warp == 0) {
         float x[12];
@@ -295,14 +353,22 @@ __global__ void __launch_bounds__(VAL_WARPS * 32, 1) k_refine_validate(DevParams
                 const long long back = total[k] - 32ll * (c - 1);
                 if (c > 0 && !done[k]) {
                     const int n = (int)(back < 32 ? back : 32);
-                    const float* o = sx + (((c - 1) & 1) * 12 * 32 + lane) * row + i;
+                    // a step a lane; without a grid the boxes of few steps
+                    // are dealt out to lanes `lanes` apart
+                    const int lanes = G.ok || n > 16 ? 32 : 1 << (32 - __clz(n - 1));
+                    const int step = lane & (lanes - 1);
+                    const float* o = sx + (((c - 1) & 1) * 12 * 32 + step) * row + i;
                     float x[12];
 #pragma unroll
                     for (int d = 0; d < 12; ++d) x[d] = o[d * 32 * row];
                     bool bad = false;
-                    if (lane < n)
-                        bad = !bounds_ok<12>(P, x) ||
-                              (V.n_obs > 0 && in_a_box<SMEM_BOXES>(P, V, s_box, G, x[0], x[1], x[2]));
+                    if (step < n) {
+                        bad = !bounds_ok<12>(P, x);
+                        if (!bad)
+                            bad = G.ok ? in_a_listed_box<SMEM_BOXES>(P, V, s_box, G, x[0], x[1], x[2])
+                                       : in_a_box<SMEM_BOXES>(V, s_box, lane / lanes, 32 / lanes, x[0], x[1], x[2]);
+                    }
+                    for (int l = lanes; l < 32; l *= 2) bad |= __shfl_xor_sync(0xFFFFFFFFu, bad, l) != 0;
                     const uint32_t b = __ballot_sync(0xFFFFFFFFu, bad);
                     if (b) {
                         done[k] = 2;
