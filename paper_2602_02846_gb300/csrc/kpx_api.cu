@@ -1495,8 +1495,10 @@ extern "C" kpx_status kpx_plan_static(const kpx_dynamics* dyn, const kpx_workspa
     int32_t left = n_iters;
     if (e == cudaSuccess && left > 0 && !(P.flags & KPX_FLAG_NO_FUSED) && fused_cluster_size(P) > 0 &&
         launch_fused(P, false, left, 0, 0, pl.stream) == cudaSuccess) {
-        if (fused_wide_size(P) > 0) e = launch_fused(P, true, -1, 0, 0, pl.stream);
-        if (e == cudaSuccess) e = sync_header();
+        // a wide form that cannot be launched leaves its iterations owed
+        if (fused_wide_size(P) > 0) launch_fused(P, true, -1, 0, 0, pl.stream);
+        cudaGetLastError();
+        e = sync_header();
         left = e == cudaSuccess ? h.graph_pending : 0;
     }
     cudaGetLastError();  // an unavailable cluster launch leaves every iteration to the phase kernels

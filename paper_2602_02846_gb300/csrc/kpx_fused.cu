@@ -26,6 +26,8 @@
 // iterations still owed to this graph launch in the header (graph_pending).
 // It then sets the graph's conditional handle, so that the loop of phase
 // kernels that follows it runs them (build_loop_graph in kpx_api.cu).
+#include <atomic>
+
 #include <cuda_runtime.h>
 
 #include "kpx_phases.cuh"
@@ -423,34 +425,39 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
     }
 }
 
+// CTAs of the form's cluster on the current device (0: unavailable), looked up
+// once per device and published whole: threads that race on the first call
+// look it up each and store the same value.
 template <int DYN, int INTEG, bool WIDE>
 int form_cluster_size() {
-    static int size = -1;
-    if (size < 0) {
-        size = 0;
-        if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-            cudaSuccess) {
-            cudaGetLastError();
-        }
-        if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FUSED_GRID_SMEM_MAX) != cudaSuccess) {
-            cudaGetLastError();
-            return size;  // 0: unavailable
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(FUSED_MAX_CLUSTER);
-        cfg.blockDim = dim3(FUSED_THREADS<DYN, WIDE>);
-        cfg.dynamicSmemBytes = FUSED_GRID_SMEM_MAX;  // the cluster must fit with a staged grid
-        int cl = 0;
-        if (cudaOccupancyMaxPotentialClusterSize(&cl, (const void*)k_fused<DYN, INTEG, WIDE>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            cl = 0;
-        }
+    constexpr int DEVICES = 64;
+    static std::atomic<int> known[DEVICES];  // the size + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (const int k = known[dev].load(std::memory_order_acquire)) return k - 1;
+    int size = 0;
+    if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess) {
+        cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(FUSED_MAX_CLUSTER);
+    cfg.blockDim = dim3(FUSED_THREADS<DYN, WIDE>);
+    cfg.dynamicSmemBytes = FUSED_GRID_SMEM_MAX;  // the cluster must fit with a staged grid
+    int cl = 0;
+    if (cudaFuncSetAttribute(k_fused<DYN, INTEG, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)FUSED_GRID_SMEM_MAX) == cudaSuccess &&
+        cudaOccupancyMaxPotentialClusterSize(&cl, (const void*)k_fused<DYN, INTEG, WIDE>, &cfg) == cudaSuccess) {
         // a power of two up to 16 (the grid is one cluster)
         int c = 1;
         while (c * 2 <= cl && c * 2 <= FUSED_MAX_CLUSTER) c *= 2;
         size = c >= 4 ? c : 0;
     }
+    cudaGetLastError();
+    known[dev].store(size + 1, std::memory_order_release);
     return size;
 }
 
