@@ -472,9 +472,9 @@ def run_kpx(args):
     value = valid_all / (ms_max / 1e3)
 
     # launches of one step (kpx_graph_info): one graph launch per kpx_iterate
-    # call, holding 1 fused launch (2 but for the quadcopter) plus 7 kernel
-    # launches per iteration the fused kernels left to the loop (begin,
-    # propagate, mark, scan, stage, append, prune); 7 per iteration without them
+    # call, holding 1 or 2 fused launches plus 7 kernel launches per iteration
+    # they left to the loop (begin, propagate, mark, scan, stage, append,
+    # prune); 7 per iteration without them, 8 without a graph
     max_g, fused = pl.graph_info()
     plan = kpx.Planner.launch_plan(iters, max_g) if max_g else [1] * iters
     pl.reset()
@@ -483,10 +483,11 @@ def run_kpx(args):
     fused_iters = int(pl.header().fused_iterations)
     graph_launches = len(plan) if max_g else 0
     if fused:
-        forms = 1 if prob.dyn == scenes.QUAD12 else 2
+        most, least = pl.layout().slot_cap, prob.lam or prob.tree_cap // 2 + 1
+        forms = 2 if prob.dyn != scenes.QUAD12 and plan[0] > 2 and least <= 512 < most else 1
         launches_per_step = 1 + forms * len(plan) + 7 * (iters - fused_iters)  # k_init (reset) first
     else:
-        launches_per_step = 1 + 7 * iters
+        launches_per_step = 1 + (7 if max_g else 8) * iters
 
     # per-phase device time over one step (same launches, CUDA events on the
     # planner's stream; nothing synchronises inside the pass, so the host

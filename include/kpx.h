@@ -254,20 +254,22 @@ kpx_status kpx_set_launch(kpx_planner* p, const kpx_launch_config* lc);
 kpx_status kpx_set_regions(kpx_planner* p, int32_t n_axes, const kpx_region_axis* axes);
 
 /* How kpx_iterate launches (the graph is built on first use): each call
- * kpx_iterate(n) is one launch of one CUDA graph per planner
+ * kpx_iterate(n) is one launch of one CUDA graph
  * (*max_iterations_per_launch = INT32_MAX; 0 when no graph can be made and
- * every iteration is eight plain launches).  The graph's first node writes
- * n into the header's graph_pending.  *fused = 1 when a fused
- * single-launch kernel follows: it runs iterations in one thread-block
- * cluster while an iteration has at most one slot per thread of the cluster
- * and the tree at most 32,768 nodes, and leaves the iterations it did not run
- * in graph_pending (the double integrator and the airplane: two such kernels,
- * the first for up to 512 slots).  A loop (a WHILE conditional node) then runs
- * seven phase kernels once per iteration left (the last block of the last
- * two counts it off graph_pending), until that is 0.  A launch of n
- * iterations thus starts 1 + 7 m kernels (2 + 7 m with two), m = the
- * iterations the fused kernels left (the header's fused_iterations counts the
- * ones they ran); without the fused kernel, 7 n. */
+ * every iteration is eight plain launches).  *fused = 1 when the graph starts
+ * with a fused single-launch kernel, n a parameter of it: it runs iterations in
+ * one thread-block cluster while an iteration has at most one slot per thread
+ * of the cluster and the tree at most 32,768 nodes, and leaves the iterations
+ * it did not run in the header's graph_pending.  The double integrator and the
+ * airplane have two such kernels, the first for up to 512 slots; a call of one
+ * or two iterations takes the first alone (up to 4,096 slots), a problem of at
+ * most 512 slots an iteration too, and one with more in every iteration
+ * (samples_per_node > 512, or 0 with a tree_cap >= 1,024) the second alone.
+ * A loop (a WHILE conditional node) then runs seven phase kernels once per
+ * iteration left (the last block of the last two counts it off graph_pending),
+ * until that is 0.  A launch of n iterations thus starts 1 + 7 m kernels
+ * (2 + 7 m with two), m = the iterations the fused kernels left (the header's
+ * fused_iterations counts the ones they ran); without the fused kernel, 7 n. */
 kpx_status kpx_graph_info(kpx_planner* p, int32_t* max_iterations_per_launch, int32_t* fused);
 
 /* Waits for the planner's stream and releases the host handle; the device

@@ -26,6 +26,15 @@ struct SideBranch {
     cudaEvent_t fork = nullptr, join = nullptr;
 };
 
+// One CUDA graph of a planner (build_loop_graph).
+struct LoopGraph {
+    cudaGraph_t graph = nullptr;  // kept: its count node is updated when n changes
+    cudaGraphExec_t exec = nullptr;
+    cudaGraphNode_t count_node = nullptr;  // holds the iteration count: the first fused kernel, or a memset
+    FusedForms forms{};
+    int32_t count = 0;  // the iterations that it is set to
+};
+
 struct kpx_planner {
     DevParams P;
     Layout L;
@@ -33,15 +42,13 @@ struct kpx_planner {
     char* ws;
     size_t ws_bytes;
     std::string err;
-    // kpx_iterate's CUDA graph (built on first use; launched on `stream`)
+    // kpx_iterate's CUDA graphs (built on first use; launched on `stream`)
     int graph_state = 0;  // 0 not decided, 1 graph, -1 unavailable (plain launches)
-    bool graph_fused = false;  // the graph starts with the fused kernel
+    bool graph_fused = false;  // the graphs start with the fused kernel
+    FusedForms forms{};        // its forms for this problem
     cudaStream_t capture_stream = nullptr;
-    SideBranch side;                       // used while capturing the loop body
-    cudaGraph_t loop_graph = nullptr;      // kept: its count node is updated before each launch
-    cudaGraphExec_t loop_exec = nullptr;
-    cudaGraphNode_t count_node = nullptr;  // memset node: the launch's iteration count
-    int32_t count_value = 1;               // the count node's current value
+    SideBranch side;           // used while capturing the loop body
+    LoopGraph loop[2];         // [1]: of calls that take one of two forms alone
     float grid_scale = GRID_SCALE_DEFAULT;  // obstacle-grid cell edge / mean box extent
     std::vector<float> host_obs; // the boxes (lo xyz, hi xyz), to rebuild the grid
     std::vector<float4> upload;  // source of kpx_create's obstacle copy, alive until destroy
@@ -378,54 +385,50 @@ cudaMemsetParams count_params(const kpx_planner* p, int n) {
     return m;
 }
 
-// kpx_iterate(n) is one launch of one graph per planner:
+// kpx_iterate(n) is one launch of one graph.  With the one-cluster kernel
+// (kpx_fused.cu):
+//   its forms (one or two), the first with n as a parameter: iterations while
+//      the problem is small; the rest stay in graph_pending
+//   -> WHILE node: kLoopIterationsFused iterations of the phase kernels per
+//      trip, until graph_pending is 0 (the end of each iteration counts it
+//      off).  The loop's handle starts at 0 and the last form sets it.
+// Without it (no forms):
 //   count node (memset: graph_pending = n)
-//   -> the fused kernel (kpx_fused.cu), when the device can run its cluster:
-//      iterations while the problem is small; the rest stay in graph_pending
-//      (two of them, the narrow and the wide form, for the double integrator
-//      and the airplane)
-//   -> WHILE node: up to kLoopIterations (kLoopIterationsFused behind the
-//      fused kernel) iterations of the phase kernels per trip, until
-//      graph_pending is 0 (each iteration's last kernel
-//      counts it off).
-// With the fused kernel the loop's handle starts at 0 and its last form
-// sets it; without it the handle starts at 1 (n >= 1).  Only the count
-// node changes between launches.
-cudaError_t build_loop_graph(kpx_planner* p, bool fused) {
+//   -> WHILE node of kLoopIterations; its handle starts at 1 (n >= 1).
+// Only the count changes between launches.
+cudaError_t build_loop_graph(const kpx_planner* p, const FusedForms& forms, int n, LoopGraph& out) {
+    const bool fused = forms.any();
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaGraphCreate(&g, 0);
     if (e != cudaSuccess) return e;
     cudaGraphConditionalHandle h = 0;
-    cudaGraphNode_t count = nullptr, dep = nullptr, loop = nullptr;
+    cudaGraphNode_t chain[2] = {}, loop = nullptr;  // the nodes in front of the loop, each behind the one before
     cudaError_t le = cudaSuccess;
     e = cudaGraphConditionalHandleCreate(&h, g, fused ? 0u : 1u, cudaGraphCondAssignDefault);
-    if (e == cudaSuccess) {
-        const cudaMemsetParams m = count_params(p, 1);
-        e = cudaGraphAddMemsetNode(&count, g, nullptr, 0, &m);
+    const int n_front = forms.both() ? 2 : 1;
+    if (e == cudaSuccess && !fused) {
+        const cudaMemsetParams m = count_params(p, n);
+        e = cudaGraphAddMemsetNode(&chain[0], g, nullptr, 0, &m);
     }
-    dep = count;
-    cudaGraphNode_t chain[3] = {count};  // the nodes so far, each behind the one before
-    const int forms = fused ? (fused_wide_size(p->P) > 0 ? 2 : 1) : 0;
-    for (int f = 0; e == cudaSuccess && f < forms; ++f) {
-        e = cudaStreamBeginCaptureToGraph(p->capture_stream, g, &dep, nullptr, 1, cudaStreamCaptureModeRelaxed);
+    for (int f = 0; e == cudaSuccess && fused && f < n_front; ++f) {
+        const bool wide = f == 1 || !forms.narrow;
+        e = cudaStreamBeginCaptureToGraph(p->capture_stream, g, f ? &chain[f - 1] : nullptr, nullptr, f ? 1 : 0,
+                                          cudaStreamCaptureModeRelaxed);
         if (e == cudaSuccess) {
-            le = launch_fused(p->P, f == 1, -1, h, f == forms - 1, p->capture_stream);
-            cudaGraph_t out = nullptr;
-            e = cudaStreamEndCapture(p->capture_stream, &out);
+            le = launch_fused(p->P, wide, fused_call(forms, wide, n, true), h, p->capture_stream);
+            cudaGraph_t same = nullptr;
+            e = cudaStreamEndCapture(p->capture_stream, &same);
             if (le != cudaSuccess) e = le;
         }
         // the captured kernel: the graph's one new node
-        cudaGraphNode_t nodes[3] = {};
-        size_t n_nodes = 3;
+        cudaGraphNode_t nodes[2] = {};
+        size_t n_nodes = 2;
         if (e == cudaSuccess) e = cudaGraphGetNodes(g, nodes, &n_nodes);
-        if (e == cudaSuccess && n_nodes != (size_t)(f + 2)) e = cudaErrorUnknown;
-        for (size_t k = 0; e == cudaSuccess && k < n_nodes; ++k) {
-            bool seen = false;
-            for (int c = 0; c <= f; ++c) seen |= nodes[k] == chain[c];
-            if (!seen) dep = chain[f + 1] = nodes[k];
-        }
-        if (e == cudaSuccess && !chain[f + 1]) e = cudaErrorUnknown;
+        if (e == cudaSuccess && n_nodes != (size_t)(f + 1)) e = cudaErrorUnknown;
+        if (e == cudaSuccess) chain[f] = f == 1 && nodes[0] != chain[0] ? nodes[0] : nodes[f];
     }
+    const cudaGraphNode_t dep = n_front > 0 ? chain[n_front - 1] : nullptr;
+    if (e == cudaSuccess && !dep) e = cudaErrorUnknown;
     cudaGraphNodeParams cp = {};
     if (e == cudaSuccess) {
         cp.type = cudaGraphNodeTypeConditional;
@@ -442,29 +445,50 @@ cudaError_t build_loop_graph(kpx_planner* p, bool fused) {
             const int unroll = fused ? kLoopIterationsFused : kLoopIterations;
             for (int u = 0; u < unroll && le == cudaSuccess; ++u)
                 le = enqueue_loop_iteration(p->P, h, u == unroll - 1, p->capture_stream, p->side);
-            cudaGraph_t out = nullptr;
-            e = cudaStreamEndCapture(p->capture_stream, &out);
+            cudaGraph_t same = nullptr;
+            e = cudaStreamEndCapture(p->capture_stream, &same);
             if (le != cudaSuccess) e = le;
         }
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&p->loop_exec, g, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&out.exec, g, 0);
     if (e != cudaSuccess) {
-        p->loop_exec = nullptr;
+        out = LoopGraph{};
         cudaGraphDestroy(g);
         return e;
     }
-    p->loop_graph = g;
-    p->count_node = count;
-    p->count_value = 1;
+    out.graph = g;
+    out.count_node = chain[0];
+    out.forms = forms;
+    out.count = n;
     return cudaSuccess;
 }
 
+// n for the next launches of a graph (a few microseconds)
+cudaError_t set_count(const kpx_planner* p, LoopGraph& g, int n) {
+    cudaError_t e = cudaSuccess;
+    if (g.forms.any()) {
+        cudaKernelNodeParams k = {};
+        e = cudaGraphKernelNodeGetParams(g.count_node, &k);  // the other parameters as captured
+        if (e != cudaSuccess) return e;
+        FusedCall call = fused_call(g.forms, !g.forms.narrow, n, true);
+        void* params[FUSED_PARAMS];
+        for (int i = 0; i < FUSED_PARAMS; ++i) params[i] = i == FUSED_CALL_PARAM ? &call : k.kernelParams[i];
+        k.kernelParams = params;
+        e = cudaGraphExecKernelNodeSetParams(g.exec, g.count_node, &k);
+    } else {
+        const cudaMemsetParams m = count_params(p, n);
+        e = cudaGraphExecMemsetNodeSetParams(g.exec, g.count_node, &m);
+    }
+    if (e == cudaSuccess) g.count = n;
+    return e;
+}
+
 void drop_graphs(kpx_planner* p) {
-    if (p->loop_exec) cudaGraphExecDestroy(p->loop_exec);
-    if (p->loop_graph) cudaGraphDestroy(p->loop_graph);
-    p->loop_exec = nullptr;
-    p->loop_graph = nullptr;
-    p->count_node = nullptr;
+    for (LoopGraph& g : p->loop) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        if (g.graph) cudaGraphDestroy(g.graph);
+        g = LoopGraph{};
+    }
 }
 
 // The stream that planners' graphs are captured on: one per host thread and
@@ -556,7 +580,7 @@ void ensure_graphs(kpx_planner* p) {
     if (p->graph_state != 0) return;
     p->graph_state = -1;
     prepare_launches(p->P);
-    p->graph_fused = !(p->P.flags & KPX_FLAG_NO_FUSED) && fused_cluster_size(p->P) > 0;
+    p->graph_fused = !(p->P.flags & KPX_FLAG_NO_FUSED) && fused_forms(p->P).any();
     cudaGetLastError();
     if (!capture_resources_here(&p->capture_stream, &p->side)) {
         p->capture_stream = nullptr;
@@ -565,16 +589,21 @@ void ensure_graphs(kpx_planner* p) {
     p->graph_state = 1;
 }
 
-// The planner's graph, built on first use (nullptr: none can be made; the
-// planner falls back to plain launches).
-cudaGraphExec_t get_graph(kpx_planner* p) {
-    if (p->loop_exec) return p->loop_exec;
+// The planner's graph for calls of n iterations, built on first use (nullptr:
+// none can be made; the planner falls back to plain launches).
+LoopGraph* get_graph(kpx_planner* p, int n) {
+    if (!p->loop[0].exec && !p->loop[1].exec) p->forms = p->graph_fused ? fused_forms(p->P) : FusedForms{};
+    const FusedForms forms = p->forms.in_call(n);
+    LoopGraph& g = p->loop[forms.both() == p->forms.both() ? 0 : 1];
+    if (g.exec) return &g;
     if (p->graph_fused) {
-        if (build_loop_graph(p, true) == cudaSuccess) return p->loop_exec;
+        if (build_loop_graph(p, forms, n, g) == cudaSuccess) return &g;
         cudaGetLastError();
+        drop_graphs(p);
         p->graph_fused = false;  // the fused form is unavailable: the phase kernels alone
+        p->forms = FusedForms{};
     }
-    if (build_loop_graph(p, false) == cudaSuccess) return p->loop_exec;
+    if (build_loop_graph(p, FusedForms{}, n, p->loop[0]) == cudaSuccess) return &p->loop[0];
     cudaGetLastError();
     p->graph_state = -1;
     return nullptr;
@@ -813,15 +842,11 @@ kpx_status kpx_iterate(kpx_planner* p, int32_t n_iters, kpx_iter_stats* out_last
     if (n_iters > 0) ensure_graphs(p);
     int32_t it = 0;
     if (p->graph_state == 1 && n_iters > 0) {
-        cudaGraphExec_t g = get_graph(p);
+        LoopGraph* g = get_graph(p, n_iters);
         if (g) {
             cudaError_t e = cudaSuccess;
-            if (n_iters != p->count_value) {  // the update costs a few microseconds: only on a change
-                const cudaMemsetParams m = count_params(p, n_iters);
-                e = cudaGraphExecMemsetNodeSetParams(g, p->count_node, &m);
-                if (e == cudaSuccess) p->count_value = n_iters;
-            }
-            if (e == cudaSuccess) e = cudaGraphLaunch(g, p->stream);
+            if (n_iters != g->count) e = set_count(p, *g, n_iters);
+            if (e == cudaSuccess) e = cudaGraphLaunch(g->exec, p->stream);
             if (e != cudaSuccess) return cuda_fail(p, e, "graph launch");
             it = n_iters;
         }
@@ -1493,15 +1518,21 @@ extern "C" kpx_status kpx_plan_static(const kpx_dynamics* dyn, const kpx_workspa
         return he == cudaSuccess ? cudaStreamSynchronize(pl.stream) : he;
     };
     int32_t left = n_iters;
-    if (e == cudaSuccess && left > 0 && !(P.flags & KPX_FLAG_NO_FUSED) && fused_cluster_size(P) > 0 &&
-        launch_fused(P, false, left, 0, 0, pl.stream) == cudaSuccess) {
-        // a wide form that cannot be launched leaves its iterations owed
-        if (fused_wide_size(P) > 0) launch_fused(P, true, -1, 0, 0, pl.stream);
+    if (e == cudaSuccess && left > 0 && !(P.flags & KPX_FLAG_NO_FUSED)) {
+        const FusedForms forms = fused_forms(P).in_call(left);
+        auto launch = [&](bool w) {
+            return launch_fused(P, w, fused_call(forms, w, left, false), 0, pl.stream) == cudaSuccess;
+        };
+        const bool narrow = forms.narrow && launch(false);
+        // behind a narrow form that runs: a wide one that cannot be launched
+        // leaves its iterations owed
+        const bool wide = forms.wide && narrow == forms.narrow && launch(true);
         cudaGetLastError();
-        e = sync_header();
-        left = e == cudaSuccess ? h.graph_pending : 0;
+        if (narrow || wide) {
+            e = sync_header();
+            left = e == cudaSuccess ? h.graph_pending : 0;
+        }
     }
-    cudaGetLastError();  // an unavailable cluster launch leaves every iteration to the phase kernels
     while (e == cudaSuccess && left > 0) {
         const int32_t n = left < kStaticIterations ? left : kStaticIterations;
         for (int32_t it = 0; e == cudaSuccess && it < n; ++it) e = enqueue_iteration(P, pl.stream);

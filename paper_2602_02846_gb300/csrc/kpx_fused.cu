@@ -55,7 +55,14 @@ namespace {
 // one alone; the double integrator at 127: 1.53 and 1.65 ms).  A growing problem
 // pays the second launch, 10 of 640 us in the double integrator's room.  The
 // quadcopter's integration costs more than its checks and needs the registers.
-constexpr int FUSED_NARROW_SLOTS = 512;
+// The second launch costs a call 2 us: a call of one or two iterations takes
+// the narrow form alone, on up to 4,096 slots (40 calls of one iteration of the
+// airplane's forest, 60 nodes: 1,039 us; both forms, the narrow one copying the
+// grid before it sees that nothing fits, 1,260; three iterations of a growing
+// tree of the airplane, past 4,096 slots: both forms 56 us a call, one 77).  A
+// problem whose slots are bounded by the line has no wide form and one whose
+// every iteration lies above it no narrow one (fused_forms()): 40 calls of the
+// double integrator at 600 slots a node 1,307 -> 1,090 us.
 template <int DYN, bool WIDE>
 constexpr int FUSED_THREADS = WIDE ? 512 : 256;
 constexpr int FUSED_MAX_PARTS = 4;
@@ -150,28 +157,37 @@ __device__ __forceinline__ void publish_iteration(const kpx_device_header* H, It
     }
 }
 
+// Iterations that the launch leaves owed when the next one does not run here: 0
+// when none is left or every further one is a no-op, all `remaining` ones when
+// it is too large; -1: it runs here.
+__device__ __forceinline__ int fused_leaves(const DevParams& P, int status, int iter, int count_A, int n_nodes,
+                                            int remaining, int max_slots) {
+    // problem_runs()
+    if (remaining <= 0 || status != KPX_OK || P.iter_limit < 0 || (P.iter_limit > 0 && iter >= P.iter_limit)) return 0;
+    const int64_t n_slots = (int64_t)count_A * begin_lambda(P, count_A);
+    return n_slots > max_slots || n_nodes > FUSED_MAX_NODES ? remaining : -1;
+}
+
+// the control word of an iteration: it runs, and needs the region snapshot
+constexpr int CTL_RUN = 1, CTL_SNAPSHOT = 2;
+
 // Leader only: decide whether the next iteration runs here; if so, begin it.
-// remaining: iterations this graph launch still owes (including this one).
-__device__ __forceinline__ void fused_begin(const DevParams& P, kpx_device_header* H, int remaining,
-                                            int64_t max_slots) {
+// remaining: iterations this graph launch still owes (including this one); the
+// header's graph_pending counts them while the launch runs.
+__device__ __forceinline__ void fused_begin(const DevParams& P, kpx_device_header* H, int remaining, int max_slots) {
+    const int left = fused_leaves(P, H->status, H->iter, H->count_A, H->n_nodes, remaining, max_slots);
     int ctl = 0;
-    if (remaining <= 0 || !problem_runs(P, H)) {
-        H->graph_pending = 0;  // done, or every further iteration is a no-op
-    } else {
-        const int64_t n_slots = (int64_t)H->count_A * begin_lambda(P, H->count_A);
-        if (n_slots > max_slots || H->n_nodes > FUSED_MAX_NODES) {
-            H->graph_pending = remaining;  // too large: the phase kernels take over
-        } else {
-            ctl = 1 | (begin_needs_snapshot(P, H) ? 2 : 0);
-            begin_counters(P, H);
-        }
+    H->graph_pending = left >= 0 ? left : remaining;
+    if (left < 0) {
+        ctl = CTL_RUN | (begin_needs_snapshot(P, H) ? CTL_SNAPSHOT : 0);
+        begin_counters(P, H);
     }
     H->graph_ctl = ctl;
 }
 
 template <int DYN, int INTEG, bool WIDE>
 __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
-    k_fused(DevParams P, int n_iter, cudaGraphConditionalHandle handle, int use_handle, int grid_smem) {
+    k_fused(DevParams P, FusedCall call, cudaGraphConditionalHandle handle, int grid_smem) {
     constexpr int THREADS = FUSED_THREADS<DYN, WIDE>, WARPS = THREADS / 32;
     extern __shared__ __align__(16) unsigned char fused_grid[];
     __shared__ uint32_t s_prefix;
@@ -193,14 +209,30 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
     __shared__ __align__(16) IterParams s_it;  // this CTA's copy of the iteration's parameters
     constexpr int HDR_WORDS = (int)(sizeof(kpx_device_header) / sizeof(uint32_t));
     static_assert(sizeof(kpx_device_header) % sizeof(uint32_t) == 0, "header size");
-    if (WIDE && P.hdr->graph_pending <= 0) {  // the narrow form left nothing (every CTA reads the same)
-        if (blockIdx.x == 0 && threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, 0u);
+    static_assert(HDR_WORDS <= THREADS, "a thread a word");
+    // the header, and the words that decide whether anything runs here, in one
+    // round trip
+    const kpx_device_header* G0 = P.hdr;
+    const int max_slots = min(call.max_slots, (int)gridDim.x * THREADS);  // a thread a slot
+    const uint32_t word0 = blockIdx.x == 0 && threadIdx.x < HDR_WORDS
+                               ? reinterpret_cast<const volatile uint32_t*>(P.hdr)[threadIdx.x]
+                               : 0u;
+    const int pending = G0->graph_pending, status = G0->status, iter0 = G0->iter, count_A = G0->count_A,
+              n_nodes = G0->n_nodes;
+    const int n_iter = call.n_iter < 0 ? pending : call.n_iter;  // < 0: what the form in front left
+    // Nothing to run here (the form in front left nothing, or the first
+    // iteration is too large): every CTA leaves at once, without the grid's
+    // copy.  They all see this: before the cluster's last barrier the header
+    // changes only here, and what the leader writes decides the same.
+    if (const int left = fused_leaves(P, status, iter0, count_A, n_nodes, n_iter, max_slots); left >= 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            P.hdr->graph_pending = left;
+            if (call.use_handle) cudaGraphSetConditional(handle, left > 0 ? 1u : 0u);
+        }
         return;
     }
     if (blockIdx.x == 0) {
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(P.hdr);
-        uint32_t* dst = reinterpret_cast<uint32_t*>(&s_hdr);
-        for (int i = threadIdx.x; i < HDR_WORDS; i += THREADS) dst[i] = src[i];
+        if (threadIdx.x < HDR_WORDS) reinterpret_cast<uint32_t*>(&s_hdr)[threadIdx.x] = word0;
         __syncthreads();
     }
     kpx_device_header* H = dsmem_generic(&s_hdr, 0);
@@ -209,7 +241,6 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
     const int n_cta = (int)gridDim.x;  // the grid is one cluster
     const int64_t gtid = (int64_t)blockIdx.x * THREADS + threadIdx.x;
     const int64_t gthreads = (int64_t)n_cta * THREADS;
-    const int64_t max_slots = WIDE || DYN == KPX_QUAD12 ? gthreads : min(gthreads, (int64_t)FUSED_NARROW_SLOTS);
     const bool early = (P.flags & KPX_FLAG_EARLY_REJECT) != 0;
     GridView G{P.cell_start, P.cell_box};
     if (grid_smem) {  // the obstacle grid is read-only while planning
@@ -223,7 +254,6 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
         __syncthreads();
         G = GridView{sc, sb};
     }
-    if (n_iter < 0) n_iter = s_hdr.graph_pending;  // read by the leader (CTA 0) only
     const bool lead_warp = blockIdx.x == 0 && threadIdx.x < 32;
     // the leader's warp keeps the books through CTA 0's own window
     kpx_device_header* HL = &s_hdr;
@@ -246,7 +276,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
         // the next iteration's while the cluster is still in this one
         const IterParams it = s_it;
         const int ctl = it.ctl;
-        if (!(ctl & 1)) break;
+        if (!(ctl & CTL_RUN)) break;
         const int64_t n_slots = it.n_slots;
         const int lam = it.lambda;
         const uint32_t iter = (uint32_t)it.iter;
@@ -254,7 +284,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
         const int32_t* va = it.va_sel ? P.va1 : P.va0;
         int32_t* va_next = it.va_sel ? P.va0 : P.va1;
         const uint32_t epoch = (uint32_t)it.epoch;
-        if (ctl & 2) {  // region snapshot for the capacity rule
+        if (ctl & CTL_SNAPSHOT) {  // region snapshot for the capacity rule
             for (int64_t r = gtid; r < P.R; r += gthreads) P.region_snap[r] = P.region_key[r];
             cluster_barrier();
         }
@@ -396,7 +426,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
             if (leader) {
                 end_counters(P, HL, false);
                 HL->fused_iterations += 1;
-                fused_begin(P, HL, n_iter - done, max_slots);
+                fused_begin(P, HL, HL->graph_pending - 1, max_slots);
             }
             publish_iteration(HL, &s_it, n_cta);
         }
@@ -405,7 +435,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
             if (leader) {
                 end_counters(P, HL, false);
                 HL->fused_iterations += 1;
-                fused_begin(P, HL, n_iter - done, max_slots);
+                fused_begin(P, HL, HL->graph_pending - 1, max_slots);
             }
             publish_iteration(HL, &s_it, n_cta);
         }
@@ -421,7 +451,7 @@ __global__ void __launch_bounds__(FUSED_THREADS<DYN, WIDE>, 1)
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&s_hdr);
         uint32_t* dst = reinterpret_cast<uint32_t*>(P.hdr);
         for (int i = threadIdx.x; i < HDR_WORDS; i += THREADS) dst[i] = src[i];
-        if (leader && use_handle) cudaGraphSetConditional(handle, s_hdr.graph_pending > 0 ? 1u : 0u);
+        if (leader && call.use_handle) cudaGraphSetConditional(handle, s_hdr.graph_pending > 0 ? 1u : 0u);
     }
 }
 
@@ -461,22 +491,23 @@ int form_cluster_size() {
     return size;
 }
 
+// The forms that a problem's iterations can use: the wide one where the slots
+// can exceed the narrow one's limit, the narrow one where they can be within
+// it.  (With lambda = 0 an iteration has more than half as many slots as the
+// tree has rows.)
 template <int DYN, int INTEG>
-int fused_cluster_size_t(const DevParams&, int) {
-    return form_cluster_size<DYN, INTEG, false>();
-}
-
-// the wide form's cluster: 0 when the system has none
-template <int DYN, int INTEG>
-int fused_wide_size_t(const DevParams&, int) {
-    if constexpr (DYN == KPX_QUAD12)
-        return 0;
-    else
-        return form_cluster_size<DYN, INTEG, true>();
+FusedForms fused_forms_t(const DevParams& P, int) {
+    FusedForms f = {form_cluster_size<DYN, INTEG, false>() > 0, false};
+    if constexpr (DYN != KPX_QUAD12) {
+        const int64_t least = P.lambda_fixed > 0 ? P.lambda_fixed : P.N / 2 + 1;
+        f.wide = P.slot_cap > FUSED_NARROW_SLOTS && form_cluster_size<DYN, INTEG, true>() > 0;
+        if (f.wide && least > FUSED_NARROW_SLOTS) f.narrow = false;
+    }
+    return f;
 }
 
 template <int DYN, int INTEG, bool WIDE>
-cudaError_t launch_form(const DevParams& P, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+cudaError_t launch_form(const DevParams& P, const FusedCall& call, cudaGraphConditionalHandle handle,
                         cudaStream_t s) {
     const int cl = form_cluster_size<DYN, INTEG, WIDE>();
     if (cl == 0) return cudaErrorNotSupported;
@@ -494,15 +525,15 @@ cudaError_t launch_form(const DevParams& P, int n_iter, cudaGraphConditionalHand
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_fused<DYN, INTEG, WIDE>, P, n_iter, handle, use_handle, grid_smem);
+    return cudaLaunchKernelEx(&cfg, k_fused<DYN, INTEG, WIDE>, P, call, handle, grid_smem);
 }
 
 template <int DYN, int INTEG>
-cudaError_t launch_fused_t(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle,
-                           int use_handle, cudaStream_t s) {
+cudaError_t launch_fused_t(const DevParams& P, bool wide, const FusedCall& call, cudaGraphConditionalHandle handle,
+                           cudaStream_t s) {
     if constexpr (DYN != KPX_QUAD12)
-        if (wide) return launch_form<DYN, INTEG, true>(P, n_iter, handle, use_handle, s);
-    return wide ? cudaErrorInvalidValue : launch_form<DYN, INTEG, false>(P, n_iter, handle, use_handle, s);
+        if (wide) return launch_form<DYN, INTEG, true>(P, call, handle, s);
+    return wide ? cudaErrorInvalidValue : launch_form<DYN, INTEG, false>(P, call, handle, s);
 }
 
 #define KPX_FUSED_DISPATCH(FN, P, ...)                                                   \
@@ -518,19 +549,23 @@ cudaError_t launch_fused_t(const DevParams& P, bool wide, int n_iter, cudaGraphC
 
 }  // namespace
 
-int fused_cluster_size(const DevParams& P) {
-    KPX_FUSED_DISPATCH(fused_cluster_size_t, P, 0);
-    return 0;
+FusedForms fused_forms(const DevParams& P) {
+    KPX_FUSED_DISPATCH(fused_forms_t, P, 0);
+    return {};
 }
 
-int fused_wide_size(const DevParams& P) {
-    KPX_FUSED_DISPATCH(fused_wide_size_t, P, 0);
-    return 0;
+FusedCall fused_call(const FusedForms& forms, bool wide, int n_iter, bool in_graph) {
+    const bool both = forms.both();
+    FusedCall c;
+    c.n_iter = wide && both ? -1 : n_iter;
+    c.max_slots = !wide && both ? FUSED_NARROW_SLOTS : INT32_MAX;
+    c.use_handle = in_graph && (wide || !both) ? 1 : 0;
+    return c;
 }
 
-cudaError_t launch_fused(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+cudaError_t launch_fused(const DevParams& P, bool wide, const FusedCall& call, cudaGraphConditionalHandle handle,
                          cudaStream_t s) {
-    KPX_FUSED_DISPATCH(launch_fused_t, P, wide, n_iter, handle, use_handle, s);
+    KPX_FUSED_DISPATCH(launch_fused_t, P, wide, call, handle, s);
     return cudaErrorInvalidValue;
 }
 

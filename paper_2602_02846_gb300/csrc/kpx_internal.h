@@ -295,17 +295,33 @@ cudaError_t launch_gather(const DevParams& P, int32_t first_row, int32_t rows, c
 // computes the cached launch shapes (SM count, occupancy) outside any capture
 void prepare_launches(const DevParams& P);
 
-// fused iterations (kpx_fused.cu): CTAs of the single cluster that runs
-// them for this problem's dynamics (0: unavailable on this device)
-int fused_cluster_size(const DevParams& P);
-// CTAs of the wide form's cluster (0: the system has none, or unavailable); it
-// goes behind the narrow one, with n_iter < 0
-int fused_wide_size(const DevParams& P);
-// up to n_iter iterations in one launch while the problem stays small
-// (n_iter < 0: the count the header's graph_pending holds at launch); the
-// rest go to the phase kernels through graph_pending and, when use_handle,
-// the graph's conditional handle (1: phase kernels needed)
-cudaError_t launch_fused(const DevParams& P, bool wide, int n_iter, cudaGraphConditionalHandle handle, int use_handle,
+// fused iterations (kpx_fused.cu): the forms of the one-cluster kernel that a
+// problem's iterations can use on the current device
+constexpr int FUSED_ALONE_ITERATIONS = 2;
+struct FusedForms {
+    bool narrow, wide;
+    bool both() const { return narrow && wide; }
+    bool any() const { return narrow || wide; }
+    // a call of few iterations takes the narrow form alone, on as many slots
+    // as it has threads
+    FusedForms in_call(int n_iter) const {
+        return both() && n_iter <= FUSED_ALONE_ITERATIONS ? FusedForms{true, false} : *this;
+    }
+};
+FusedForms fused_forms(const DevParams& P);
+constexpr int FUSED_NARROW_SLOTS = 512;  // slots of the iterations that the narrow form takes in front of the wide one
+// what one launch of a form does (the kernel's second parameter)
+struct FusedCall {
+    int32_t n_iter;      // iterations at most (< 0: the count the header's graph_pending holds at launch)
+    int32_t max_slots;   // slots of an iteration it takes
+    int32_t use_handle;  // sets the graph's conditional handle (1: phase kernels needed)
+};
+constexpr int FUSED_CALL_PARAM = 1, FUSED_PARAMS = 4;
+// a form's part in a call of n_iter iterations by `forms`
+FusedCall fused_call(const FusedForms& forms, bool wide, int n_iter, bool in_graph);
+// iterations in one launch while the problem stays small; the rest go to the
+// wide form or the phase kernels through graph_pending
+cudaError_t launch_fused(const DevParams& P, bool wide, const FusedCall& call, cudaGraphConditionalHandle handle,
                          cudaStream_t s);
 
 // trajectory refinement (kpx_adjoint.cu: objective, adjoint gradient and
