@@ -518,7 +518,8 @@ extern "C" kpx_status kpx_refine_validate(const kpx_dynamics* dyn, const kpx_wor
     if (smem_boxes) smem += boxes;
     const auto kernel = P.iso_inertia ? (smem_boxes ? k_refine_validate<true, true> : k_refine_validate<true, false>)
                                       : (smem_boxes ? k_refine_validate<false, true> : k_refine_validate<false, false>);
-    if (allow_smem((const void*)kernel, smem) != cudaSuccess) return KPX_E_CUDA;
+    static std::atomic<uint64_t> done[2][2];
+    if (allow_smem((const void*)kernel, smem, done[P.iso_inertia ? 1 : 0][smem_boxes]) != cudaSuccess) return KPX_E_CUDA;
     kernel<<<(count + per_block - 1) / per_block, VAL_WARPS * 32, smem, reinterpret_cast<cudaStream_t>(cuda_stream)>>>(
         P, V, per_block, row);
     return cudaGetLastError() == cudaSuccess ? KPX_OK : KPX_E_CUDA;

@@ -5,6 +5,7 @@
 // (int32[count][max_segments]) and max_segments.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -64,20 +65,34 @@ __device__ __forceinline__ void feed_steps(const Params& R, int64_t tr, int S, i
 
 // Dynamic shared memory that a refinement kernel may be launched with: the
 // 227 KB of a block less 1 KB for the kernels' static arrays.  The limit belongs
-// to the function, not to the launch, so every caller sets this same value: one
-// that set its own call's size could lower it under another thread's launch.
+// to the function, not to the launch, so it is set to this same value by every
+// caller (one that set its own call's size could lower it under another
+// thread's launch), and once per device: `done` holds a bit for each.  (Each
+// call setting it cost 2 us of host time.)
 constexpr size_t REFINE_SMEM_MAX = 226 * 1024;
 
-inline cudaError_t allow_smem(const void* fn, size_t bytes) {
+inline cudaError_t allow_smem(const void* fn, size_t bytes, std::atomic<uint64_t>& done) {
     if (bytes > REFINE_SMEM_MAX) return cudaErrorInvalidValue;
     if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REFINE_SMEM_MAX);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;  // 0: set at every call
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REFINE_SMEM_MAX);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
 }
 
 inline int device_sms() {
+    static std::atomic<int> known[64];
     int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    const bool keep = dev >= 0 && dev < 64;
+    if (keep) sms = known[dev].load(std::memory_order_relaxed);
+    if (sms > 0) return sms;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (keep && sms > 0) known[dev].store(sms, std::memory_order_relaxed);
     return sms > 0 ? sms : 1;
 }
 
