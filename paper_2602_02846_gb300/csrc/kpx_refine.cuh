@@ -67,13 +67,13 @@ __device__ __forceinline__ void feed_steps(const Params& R, int64_t tr, int S, i
 // 227 KB of a block less 1 KB for the kernels' static arrays.  The limit belongs
 // to the function, not to the launch, so it is set to this same value by every
 // caller (one that set its own call's size could lower it under another
-// thread's launch), and once per device: `done` holds a bit for each.  (Each
-// call setting it cost 2 us of host time.)
+// thread's launch), whatever this call's (the default of 48 KB is for dynamic
+// and static shared memory together), and once per device: `done` holds a bit
+// for each.  (Each call setting it cost 2 us of host time.)
 constexpr size_t REFINE_SMEM_MAX = 226 * 1024;
 
 inline cudaError_t allow_smem(const void* fn, size_t bytes, std::atomic<uint64_t>& done) {
     if (bytes > REFINE_SMEM_MAX) return cudaErrorInvalidValue;
-    if (bytes <= 48 * 1024) return cudaSuccess;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
