@@ -128,18 +128,20 @@ __global__ void k_init(DevParams P, int first_time) {
 // obstacle grid (broad phase), built once per create: each cell lists its
 // boxes in ascending box index.
 //
-// One launch: a block takes GRID_CELLS_PER_BLOCK consecutive cells.  A box
+// One launch: a block takes GRID_THREADS / PARTS consecutive cells.  A box
 // covers a box of cells, so how many of its cells lie before the block's first
 // one has a closed form, and the sum over the boxes is where the block's lists
 // start: no counting pass and no scan over the cells.  The block then keeps
-// the boxes that meet its rows of cells (in order, by ballots), and four
-// threads a cell count and copy a quarter of those each.  Bound: launch latency
+// the boxes that meet its rows of cells (in order, by ballots), and PARTS
+// threads a cell count and copy as many parts of those.  Bound: launch latency
 // and three passes over the boxes from L2.  (A warp per cell over every box, twice, and a scan
 // by one block took 85 us for 1,000 boxes and 41,472 cells; this takes under 15 us.)
+// PARTS is 4 while that gives every SM a block, else 32: large boxes make few
+// cells with long lists (creating a planner with 1,000 boxes half as wide as the
+// workspace: 177 us with 4, 101 with 32; 127 with a warp per cell as above; with
+// 6,000 boxes 848, 386 and 386).
 // ---------------------------------------------------------------------------
 constexpr int GRID_THREADS = 256;
-constexpr int GRID_PARTS = 4;  // threads a cell
-constexpr int GRID_CELLS_PER_BLOCK = GRID_THREADS / GRID_PARTS;
 
 // the cell range of box b: lo x, y, z, hi x, y, z
 __device__ __forceinline__ void box_range(const DevParams& P, int b, int (&r)[6]) {
@@ -152,15 +154,17 @@ __device__ __forceinline__ void box_range(const DevParams& P, int b, int (&r)[6]
     }
 }
 
+template <int PARTS>
 __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
+    constexpr int CELLS = GRID_THREADS / PARTS;
     constexpr int LIST = 1024;  // boxes listed at a time
     __shared__ uint32_t s_warp[GRID_THREADS / 32];
     __shared__ uint16_t s_box[LIST];
     __shared__ uint32_t s_lo[LIST], s_hi[LIST];  // their ranges, a byte an axis
     static_assert(GRID_MAX_AXIS <= 256, "a cell index fits a byte");
     const int nx = P.grid_n[0], ny = P.grid_n[1];
-    const int c0 = blockIdx.x * GRID_CELLS_PER_BLOCK;
-    const int c1 = min(c0 + GRID_CELLS_PER_BLOCK, P.n_cells) - 1;  // the block's last cell
+    const int c0 = blockIdx.x * CELLS;
+    const int c1 = min(c0 + CELLS, P.n_cells) - 1;  // the block's last cell
     const int fx = c0 % nx, fy = c0 / nx % ny, fz = c0 / (nx * ny);
     const int ly = c1 / nx % ny, lz = c1 / (nx * ny);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -189,7 +193,7 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
             P.hdr->err_info[2] = total;
         }
     }
-    const int c = c0 + (int)threadIdx.x / GRID_PARTS, part = (int)threadIdx.x % GRID_PARTS;
+    const int c = c0 + (int)threadIdx.x / PARTS, part = (int)threadIdx.x % PARTS;
     const uint32_t cx = (uint32_t)(c % nx), cy = (uint32_t)(c / nx % ny), cz = (uint32_t)(c / (nx * ny));
     uint32_t at_cell = 0;  // pass 1: the cell's next entry
     for (int pass = 0; pass < 2; ++pass) {  // count, then copy
@@ -221,8 +225,8 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
                 }
                 __syncthreads();
             }
-            // this thread's quarter of the list
-            const int l0 = listed * part / GRID_PARTS, l1 = listed * (part + 1) / GRID_PARTS;
+            // this thread's part of the list
+            const int l0 = listed * part / PARTS, l1 = listed * (part + 1) / PARTS;
             auto lists = [&](int l) {
                 const uint32_t lo = s_lo[l], hi = s_hi[l];
                 return cx >= (lo & 255u) && cx <= (hi & 255u) && cy >= (lo >> 8 & 255u) && cy <= (hi >> 8 & 255u) &&
@@ -232,11 +236,11 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
             for (int l = l0; l < l1; ++l) k += lists(l) ? 1u : 0u;
             n += k;
             if (pass == 1) {
-                // the quarters in order, behind the cell's entries of earlier lists
+                // the parts in order, behind the cell's entries of earlier lists
                 uint32_t upto = k;
 #pragma unroll
-                for (int o = 1; o < GRID_PARTS; o <<= 1) {
-                    const uint32_t y = __shfl_up_sync(FULL, upto, o, GRID_PARTS);
+                for (int o = 1; o < PARTS; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(FULL, upto, o, PARTS);
                     if (part >= o) upto += y;
                 }
                 uint32_t at = at_cell + upto - k;
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
                         }
                         ++at;
                     }
-                at_cell += __shfl_sync(FULL, upto, GRID_PARTS - 1, GRID_PARTS);
+                at_cell += __shfl_sync(FULL, upto, PARTS - 1, PARTS);
             }
             __syncthreads();  // the list is rewritten for the next boxes, or the next pass
         }
@@ -257,8 +261,8 @@ __global__ void __launch_bounds__(GRID_THREADS) k_grid_build(DevParams P) {
             uint32_t sum;
             if (c > c1) n = 0;
             const uint32_t pos = start + block_exclusive_scan<GRID_THREADS>(n, sum, s_warp);
-            at_cell = __shfl_sync(FULL, pos, 0, GRID_PARTS);
-            const uint32_t end = __shfl_sync(FULL, pos + n, GRID_PARTS - 1, GRID_PARTS);
+            at_cell = __shfl_sync(FULL, pos, 0, PARTS);
+            const uint32_t end = __shfl_sync(FULL, pos + n, PARTS - 1, PARTS);
             if (c <= c1 && part == 0) {
                 P.cell_start[c] = (int32_t)at_cell;
                 P.cell_pair[c] = make_int2((int32_t)at_cell, (int32_t)min(end, (uint32_t)P.grid_cap));
@@ -680,7 +684,11 @@ cudaError_t launch_init(const DevParams& P, bool first_time, cudaStream_t s) {
 
 cudaError_t launch_grid_build(const DevParams& P, cudaStream_t s) {
     if (P.n_obs == 0) return cudaSuccess;
-    k_grid_build<<<(P.n_cells + GRID_CELLS_PER_BLOCK - 1) / GRID_CELLS_PER_BLOCK, GRID_THREADS, 0, s>>>(P);
+    const auto blocks = [&](int cells) { return (P.n_cells + cells - 1) / cells; };
+    if (blocks(GRID_THREADS / 4) >= sm_count())
+        k_grid_build<4><<<blocks(GRID_THREADS / 4), GRID_THREADS, 0, s>>>(P);
+    else
+        k_grid_build<32><<<blocks(GRID_THREADS / 32), GRID_THREADS, 0, s>>>(P);
     return cudaGetLastError();
 }
 
