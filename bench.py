@@ -56,7 +56,7 @@ SM_COUNT_FALLBACK = 152
 # DRAM bytes (read + write) of one propagate launch from the ncu captures in
 # profiles/ (the kernel build named there); None for a workload not captured.
 FUSED_DRAM_BYTES = {
-    "dubins6_forest300": 195072,     # profiles/k_fused_dubins6_forest300.md (the timed step's graph launch)
+    "dubins6_forest300": 284160,     # profiles/k_fused_dubins6_forest300.md (the timed step's graph launch)
 }
 PROPAGATE_DRAM_BYTES = {
     "quad12_building1000": 6868736,  # profiles/k_propagate_quad12_building1000.md (iteration 100)
@@ -1044,7 +1044,7 @@ def run_refine(args):
                          **fma_fields(achieved),
                          "forward_only_ms": fwd_ms, "forward_and_backward_ms": both_ms},
             "cpu_baseline": cpu, "e2e": e2e, "clocks": clk,
-            "gpu_launches": 2 * args.steps,
+            "gpu_launches": 5 * args.steps,  # the box grid's three, forward, backward
         }
         print(json.dumps(line))
     return 0
