@@ -484,7 +484,7 @@ def run_kpx(args):
     graph_launches = len(plan) if max_g else 0
     if fused:
         most, least = pl.layout().slot_cap, prob.lam or prob.tree_cap // 2 + 1
-        forms = 2 if prob.dyn != scenes.QUAD12 and plan[0] > 2 and least <= 512 < most else 1
+        forms = 2 if prob.dyn != scenes.QUAD12 and least <= 512 < most else 1
         launches_per_step = 1 + forms * len(plan) + 7 * (iters - fused_iters)  # k_init (reset) first
     else:
         launches_per_step = 1 + (7 if max_g else 8) * iters

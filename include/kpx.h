@@ -254,17 +254,18 @@ kpx_status kpx_set_launch(kpx_planner* p, const kpx_launch_config* lc);
 kpx_status kpx_set_regions(kpx_planner* p, int32_t n_axes, const kpx_region_axis* axes);
 
 /* How kpx_iterate launches (the graph is built on first use): each call
- * kpx_iterate(n) is one launch of one CUDA graph
+ * kpx_iterate(n) is one launch of one CUDA graph of the planner's
  * (*max_iterations_per_launch = INT32_MAX; 0 when no graph can be made and
  * every iteration is eight plain launches).  *fused = 1 when the graph starts
  * with a fused single-launch kernel, n a parameter of it: it runs iterations in
  * one thread-block cluster while an iteration has at most one slot per thread
  * of the cluster and the tree at most 32,768 nodes, and leaves the iterations
  * it did not run in the header's graph_pending.  The double integrator and the
- * airplane have two such kernels, the first for up to 512 slots; a call of one
- * or two iterations takes the first alone (up to 4,096 slots), a problem of at
- * most 512 slots an iteration too, and one with more in every iteration
- * (samples_per_node > 512, or 0 with a tree_cap >= 1,024) the second alone.
+ * airplane have two such kernels, the first for up to 512 slots; a problem of
+ * at most 512 slots an iteration takes the first alone, one with more in every
+ * iteration (samples_per_node > 512, or 0 with a tree_cap >= 1,024) the second
+ * alone, and a planner that has made 64 calls of one or two iterations takes
+ * the first alone in further such calls (up to 4,096 slots).
  * A loop (a WHILE conditional node) then runs seven phase kernels once per
  * iteration left (the last block of the last two counts it off graph_pending),
  * until that is 0.  A launch of n iterations thus starts 1 + 7 m kernels

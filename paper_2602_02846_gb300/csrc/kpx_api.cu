@@ -49,6 +49,7 @@ struct kpx_planner {
     cudaStream_t capture_stream = nullptr;
     SideBranch side;           // used while capturing the loop body
     LoopGraph loop[2];         // [1]: of calls that take one of two forms alone
+    int few_calls = 0;         // calls that would have, before it is built (-1: it cannot be)
     float grid_scale = GRID_SCALE_DEFAULT;  // obstacle-grid cell edge / mean box extent
     std::vector<float> host_obs; // the boxes (lo xyz, hi xyz), to rebuild the grid
     std::vector<float4> upload;  // source of kpx_create's obstacle copy, alive until destroy
@@ -589,21 +590,34 @@ void ensure_graphs(kpx_planner* p) {
     p->graph_state = 1;
 }
 
+// A graph costs 100 us of host time to build, the second form 2 us a call: the
+// graph of the calls that go without it is built only for a planner that has
+// made this many of them (one iteration and then 100 on a new planner: 1,017 us
+// with one graph, 1,097 with both).
+constexpr int kFewCalls = 64;
+
 // The planner's graph for calls of n iterations, built on first use (nullptr:
 // none can be made; the planner falls back to plain launches).
 LoopGraph* get_graph(kpx_planner* p, int n) {
-    if (!p->loop[0].exec && !p->loop[1].exec) p->forms = p->graph_fused ? fused_forms(p->P) : FusedForms{};
-    const FusedForms forms = p->forms.in_call(n);
-    LoopGraph& g = p->loop[forms.both() == p->forms.both() ? 0 : 1];
-    if (g.exec) return &g;
+    LoopGraph& whole = p->loop[0];
+    LoopGraph& alone = p->loop[1];
+    if (!whole.exec) p->forms = p->graph_fused ? fused_forms(p->P) : FusedForms{};
+    if (p->forms.both() && !p->forms.in_call(n).both()) {
+        if (!alone.exec && p->few_calls >= 0 && ++p->few_calls > kFewCalls &&
+            build_loop_graph(p, p->forms.in_call(n), n, alone) != cudaSuccess) {
+            cudaGetLastError();
+            p->few_calls = -1;  // no second graph
+        }
+        if (alone.exec) return &alone;
+    }
+    if (whole.exec) return &whole;
     if (p->graph_fused) {
-        if (build_loop_graph(p, forms, n, g) == cudaSuccess) return &g;
+        if (build_loop_graph(p, p->forms, n, whole) == cudaSuccess) return &whole;
         cudaGetLastError();
-        drop_graphs(p);
         p->graph_fused = false;  // the fused form is unavailable: the phase kernels alone
         p->forms = FusedForms{};
     }
-    if (build_loop_graph(p, FusedForms{}, n, p->loop[0]) == cudaSuccess) return &p->loop[0];
+    if (build_loop_graph(p, FusedForms{}, n, whole) == cudaSuccess) return &whole;
     cudaGetLastError();
     p->graph_state = -1;
     return nullptr;

@@ -55,8 +55,9 @@ namespace {
 // one alone; the double integrator at 127: 1.53 and 1.65 ms).  A growing problem
 // pays the second launch, 10 of 640 us in the double integrator's room.  The
 // quadcopter's integration costs more than its checks and needs the registers.
-// The second launch costs a call 2 us: a call of one or two iterations takes
-// the narrow form alone, on up to 4,096 slots (40 calls of one iteration of the
+// The second launch costs a call 2 us: calls of one or two iterations, once a
+// planner has made many (get_graph() in kpx_api.cu), take the narrow form alone,
+// on up to 4,096 slots (40 calls of one iteration of the
 // airplane's forest, 60 nodes: 1,039 us; both forms, the narrow one copying the
 // grid before it sees that nothing fits, 1,260; three iterations of a growing
 // tree of the airplane, past 4,096 slots: both forms 56 us a call, one 77).  A

@@ -19,9 +19,14 @@ from tests.test_gpu_fused import _same, _state  # noqa: E402
     (scenes.di_scene, 0, 900), (scenes.di_scene, 0, 1023), (scenes.dubins_scene, 0, 1024), (scenes.di_scene, 0, 5000),
 ])
 @pytest.mark.parametrize("calls", [(1,), (2, 1), (3, 1, 40, 2)])
-def test_calls_equal_phase_kernels(make, lam, cap, calls):
+@pytest.mark.parametrize("many", [False, True])
+def test_calls_equal_phase_kernels(make, lam, cap, calls, many):
     prob = make(5, n_obstacles=40, tree_cap=cap, lam=lam)
     fused, plain = kpx.Planner(prob), kpx.Planner(prob, flags=kpx.KPX_FLAG_NO_FUSED)
+    if many:  # the graph of the few-iteration calls is built after 64 of them
+        for _ in range(70):
+            fused.iterate(1)
+        fused.reset()
     for i in range(60 // sum(calls) + 1):
         for n in calls:
             fused.iterate(n)
